@@ -286,6 +286,15 @@ def insert_launches(api, h, n: int) -> int:
     return 3 if blocked else 1
 
 
+def lookup_launches(api, h, n: int) -> int:
+    """Kernels one wc_retrieve launches (4 for the region-split scheme, else 1)."""
+    lc = api.wc_table_get_launch(h, 1)
+    info = api.wc_table_get_info(h)
+    blocked = lc["scheme"] == 2 or (lc["scheme"] == 0 and info["table_bytes"] > (512 << 20)
+                                     and n >= info["table_bytes"] // 64)
+    return 4 if blocked else 1
+
+
 def timed(s, f):
     """Run f() between two events on stream s; returns ms."""
     import torch
@@ -501,7 +510,7 @@ def run_wc(args, rank, world, local_rank):
                    "group_retrieve": g_ret,
                    "insert_keys_in_flight": api.wc_table_get_launch(h, wc.WC_OP_INSERT)["keys_in_flight"],
                    "retrieve_keys_in_flight": api.wc_table_get_launch(h, wc.WC_OP_RETRIEVE)["keys_in_flight"],
-                   "retrieve_scheme": {0: "auto (direct)", 1: "direct", 2: "region split", 3: "grouped duplicates"}[
+                   "retrieve_scheme": {0: "auto", 1: "direct", 2: "region split", 3: "grouped duplicates"}[
                        api.wc_table_get_launch(h, wc.WC_OP_RETRIEVE)["scheme"]],
                    "table_bytes": info["table_bytes"], "overflow_bits": bool(info["options"] & 1),
                    "layout": "struct of arrays" if info["options"] & 2 else "packed 64-bit slots",
@@ -522,7 +531,7 @@ def run_wc(args, rank, world, local_rank):
                      # a random miss fills a whole 128-byte L2 line (measured with the library's
                      # random-access probe): the traffic in lines per operation
                      "dram_lines_per_op": None if traffic is None else traffic / 128 / n},
-        "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (insert_launches(api, h, n) + 1) * args.steps,
+        "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": (insert_launches(api, h, n) + lookup_launches(api, h, n)) * args.steps,
         "clocks": clk.summary(),
     }
     if args.alphas:
@@ -723,7 +732,7 @@ def run_sv64_zipf(args, dev):
                  op: {k: lc_[k] for k in ("group_size", "keys_in_flight", "scheme")}
                  for op, lc_ in (("insert", api.wc_table_get_launch(h, wc.WC_OP_INSERT)), ("retrieve", lc))},
              "l2": "no flush: table 4.8 GB"}, clk,
-            (insert_launches(api, h, n) + 1) * args.steps,
+            (insert_launches(api, h, n) + lookup_launches(api, h, n)) * args.steps,
             {"insert_gops": n / ins / 1e6, "retrieve_gops": n / ret / 1e6, "insert_ms": ins, "retrieve_ms": ret,
              "retrieve_dedup_gops": n / ret_dedup / 1e6, "retrieve_dedup_ms": ret_dedup,
              "roofline": {"bound": "hbm", "kernel": "k_sv_retrieve", "achieved": 48 * n / (ret * 1e-3) / 1e9,

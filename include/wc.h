@@ -197,7 +197,9 @@ typedef struct {
  * keys_in_flight = keys each group probes at once (1 or 2; 0 = 1): with 2, every trip of
  * a group loads the windows of two keys, so twice as many random window reads are in
  * flight per warp (single-value retrieves of up to 32 bytes of window per lane; elsewhere
- * it is taken as 1).  Default 2 for lookups of 4+4-byte single-value tables, else 1. */
+ * it is taken as 1).  Default 2 for lookups of 4+4-byte single-value tables, else 1.
+ * Lookups of windows of at most 64 bytes run one query per thread, whatever group_size,
+ * block_threads, blocks_per_sm and keys_in_flight say (WC_SCHEME_DEDUP keeps the group). */
 typedef struct {
   int32_t group_size;
   int32_t block_threads;
@@ -210,12 +212,16 @@ typedef struct {
 /* WC_SCHEME_DIRECT: every key probes the table where its hash points, in input order.
  * WC_SCHEME_BLOCKED: the batch is first split by table region (the multi-split of
  * Sec. IV-E applied to regions of one table) and then probed region by region, so the
- * active part of the table stays in L2; needs scratch of n * (key + value) bytes, which
- * the table allocates on first use (stream-ordered) and keeps.  Inserts of single-value,
+ * active part of the table stays in L2; needs scratch of n * (key + value) bytes (lookups:
+ * n * (key + value + 3) bytes and 8 bytes per 4096 queries and region), which the table
+ * allocates on first use (stream-ordered) and keeps; calls that share it on different
+ * streams are ordered one behind the other.  Inserts of single-value,
  * counting, hash-set and open-addressing multi-value tables; retrieves of single-value and
- * counting tables (the results are split back into input order).  WC_SCHEME_AUTO picks
+ * counting tables (the results are put back in input order).  WC_SCHEME_AUTO picks
  * BLOCKED for those inserts when the batch holds at least 2^18 pairs and the table is
- * larger than 64 MiB, DIRECT otherwise.
+ * larger than 64 MiB, for lookups (wc_retrieve, wc_contains; hash sets too) when the slots
+ * take more than 512 MiB and the batch holds at least one query per 64 bytes of them (and
+ * the stream is not being captured and the scratch fits), DIRECT otherwise.
  * WC_SCHEME_DEDUP (lookups of single-value, counting and hash-set tables: wc_retrieve,
  * wc_contains): direct probing, but equal keys among each 32 consecutive queries of a
  * warp are found with one warp vote (__match_any_sync) and probed once, the result written

@@ -240,7 +240,20 @@ int occupancy_cached(const void* kernel, int block, size_t smem) {
   return nb;
 }
 
-cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s) {
+bool stream_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, uint64_t likely) {
+  if (t->scratch_ev != nullptr && t->scratch_stream != s && !stream_capturing(s)) {
+    const cudaError_t e = cudaStreamWaitEvent(s, t->scratch_ev, 0);
+    if (e != cudaSuccess) return e;
+  }
   if (bytes <= t->scratch_bytes) return cudaSuccess;
   if (t->d_scratch != nullptr) {
     cudaError_t e = cudaFreeAsync(t->d_scratch, s);
@@ -248,15 +261,58 @@ cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s) {
     t->d_scratch = nullptr;
     t->scratch_bytes = 0;
   }
-  const uint64_t want = align_up(bytes + bytes / 8, kAlign);
   if (injected_alloc_failure()) return cudaErrorMemoryAllocation;
+  uint64_t want = align_up(std::max(bytes + bytes / 8, likely), kAlign);
   cudaError_t e = cudaMallocAsync(&t->d_scratch, want, s);
+  if (e == cudaErrorMemoryAllocation && want > align_up(bytes, kAlign)) {
+    cudaGetLastError();  // no room for more than this call needs
+    want = align_up(bytes, kAlign);
+    e = cudaMallocAsync(&t->d_scratch, want, s);
+  }
   if (e != cudaSuccess) {
     t->d_scratch = nullptr;
     return e;
   }
   t->scratch_bytes = want;
   return cudaSuccess;
+}
+
+cudaError_t scratch_release(const wc_table* t, cudaStream_t s) {
+  if (stream_capturing(s)) return cudaSuccess;
+  if (t->scratch_ev == nullptr) {
+    const cudaError_t e = cudaEventCreateWithFlags(&t->scratch_ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+  }
+  t->scratch_stream = s;
+  return cudaEventRecord(t->scratch_ev, s);
+}
+
+// Lookups split by region where the table is far larger than L2 and the batch asks for each
+// of its 64-byte windows about once: the split costs ~9 ps a query (4-byte keys) and one
+// sequential pass over the table, and saves a random HBM line per query.  4+4-byte pairs at
+// load 0.9, half the queries absent, direct against split: 1.1 GiB table 28.5 against 46.3
+// G lookups/s for 2^27 queries, 27.8 against 30.1 for 2^24, 17.9 against 11.6 for 2^20;
+// 2 GiB table at load 0.5 37.0 against 34.2 for 2^24.  Between L2's size and 512 MiB the split
+// still wins on uniform queries (284 MiB, 2^26: 40.0 against 49.2) but loses on skewed ones,
+// whose hot lines stay in L2 (256 MiB, Zipf: 78 against 49); above, it wins both (1.1 GiB,
+// Zipf: 32.5 against 48.1).  8+8-byte pairs: 2.2 GiB 23.8 against 27.1, Zipf 28.8 against
+// 35.8.  Not inside a stream capture: the scratch must not belong to the graph.
+static bool lookup_splits(const wc_table* t, uint64_t n) {
+  return t->table_bytes > (512ull << 20) && n >= t->table_bytes / 64;
+}
+
+int lookup_scheme(const wc_table* t, uint64_t n, cudaStream_t s) {
+  const int sc = t->launch[WC_OP_RETRIEVE].scheme;
+  if (sc != WC_SCHEME_AUTO) return sc;
+  return lookup_splits(t, n) && !stream_capturing(s) ? WC_SCHEME_BLOCKED : WC_SCHEME_DIRECT;
+}
+
+uint64_t lookup_scratch_likely(const wc_table* t, uint64_t n) {
+  if (t->cfg.kind != WC_SINGLE_VALUE && t->cfg.kind != WC_COUNTING && t->cfg.kind != WC_HASH_SET) return 0;
+  const int sc = t->launch[WC_OP_RETRIEVE].scheme;
+  if (sc != WC_SCHEME_BLOCKED && !(sc == WC_SCHEME_AUTO && lookup_splits(t, n))) return 0;
+  // keys, positions in their tile, values, found bytes; run starts per tile of 4096 and region
+  return n * (2 * static_cast<uint64_t>(t->cfg.key_bytes) + 3) + (n / 512 + 8) * (t->table_bytes / (16ull << 20) + 2) + (1ull << 16);
 }
 
 int scheme_for(const wc_table* t, int op, uint64_t n) {
@@ -547,6 +603,7 @@ wc_status wc_table_destroy(wc_table* t) {
     cudaDeviceSynchronize();
     cudaFree(t->d_scratch);
   }
+  if (t->scratch_ev != nullptr) cudaEventDestroy(t->scratch_ev);
   cudaError_t e = cudaFree(t->d_block);
   delete t;
   return cuda_status(e);

@@ -173,7 +173,9 @@ cudaError_t count_insert(const wc_table* t, const void* keys, const void* weight
   cudaError_t e = kb == 4 ? aggregate<uint32_t, uint32_t>(t, keys, weights, n, skip, &ak, &av, s)
                           : aggregate<unsigned long long, unsigned long long>(t, keys, weights, n, skip, &ak, &av, s);
   if (e != cudaSuccess) return e;
-  return count_insert_agg(t, ak, av, n, s);
+  e = count_insert_agg(t, ak, av, n, s);
+  const cudaError_t r = scratch_release(t, s);
+  return e != cudaSuccess ? e : r;
 }
 
 }  // namespace wc

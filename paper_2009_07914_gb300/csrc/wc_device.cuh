@@ -70,7 +70,7 @@ __device__ __forceinline__ void load_words(const unsigned long long* p, unsigned
 // batches flowing through L2 displace table lines as little as possible.
 __device__ __forceinline__ unsigned long long evict_first_policy() {
   unsigned long long pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
 __device__ __forceinline__ uint32_t ldg_stream(const uint32_t* p) {
@@ -106,7 +106,7 @@ __device__ __forceinline__ unsigned long long ldg_stream(const unsigned long lon
 // gain (6.9 -> 6.4 G inserts/s with the hint).
 __device__ __forceinline__ unsigned long long evict_last_policy() {
   unsigned long long pol;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+  asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
 __device__ __forceinline__ uint32_t ovf_word(const uint32_t* ovf, uint32_t w) {

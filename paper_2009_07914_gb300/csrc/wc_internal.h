@@ -142,6 +142,8 @@ struct wc_table {
   // scratch for the blocked scheme, grown on demand (stream-ordered allocation)
   mutable void* d_scratch;
   mutable uint64_t scratch_bytes;
+  mutable cudaEvent_t scratch_ev = nullptr;  // end of the last call that used the scratch
+  mutable cudaStream_t scratch_stream = nullptr;  // and its stream
   wc::HostPipe* host = nullptr;  // host-buffer pipeline, created on first use
 };
 
@@ -172,8 +174,16 @@ uint64_t scan_partials_needed(uint64_t n);
 
 int sm_count_of(int device);
 
-// Scratch of at least `bytes` on stream s (grows the table's buffer if needed).
-cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s);
+// Scratch of at least `bytes` on stream s (grows the table's buffer if needed), ordered
+// behind the last call that used it: calls of the same kind may overlap on different
+// streams, and there is one buffer per table.  scratch_release marks the end of this call's
+// use of it (after its last kernel).  Inside a stream capture neither touches the event.
+// likely: bytes that calls expected next will need, taken along when the buffer grows.
+cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, uint64_t likely = 0);
+cudaError_t scratch_release(const wc_table* t, cudaStream_t s);
+
+// Whether s is being captured into a graph.
+bool stream_capturing(cudaStream_t s);
 
 // Release the table's host-buffer pipeline (streams, events, staging).
 void host_pipe_free(wc_table* t);
@@ -188,5 +198,12 @@ bool autotune_enabled();
 
 // Scheme the table uses for `op` on a batch of n keys.
 int scheme_for(const wc_table* t, int op, uint64_t n);
+
+// The same for lookups, on stream s.
+int lookup_scheme(const wc_table* t, uint64_t n, cudaStream_t s);
+
+// Scratch a split lookup of n queries takes (0: it would not be split): an insert of as
+// many pairs grows the buffer to it, so the lookup after it does not have to grow it again.
+uint64_t lookup_scratch_likely(const wc_table* t, uint64_t n);
 
 }  // namespace wc

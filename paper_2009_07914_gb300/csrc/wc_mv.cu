@@ -67,7 +67,9 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
   e = launch_k(t, t->growth == kGrowExact ? k_mv_alloc<VB> : k_mv_alloc_growth<VB>, g_a, kAllocThreads, 0, s, d, pd,
                t->capacity);
   if (e != cudaSuccess) return e;
-  return launch_k(t, place, g_p, kThreads, 0, s, d, pd, rec, vals, n, counters ? counters + 1 : counters);
+  e = launch_k(t, place, g_p, kThreads, 0, s, d, pd, rec, vals, n, counters ? counters + 1 : counters);
+  const cudaError_t r = scratch_release(t, s);
+  return e != cudaSuccess ? e : r;
 }
 
 // The aggregation passes run blocks of the insert launch's block_threads (256 or 512;

@@ -29,7 +29,9 @@ cudaError_t oa_run(const wc_table* t, int op, const void* keys, const void* vals
     cudaError_t e = region_split(t, lc.region_mib, k, static_cast<const Val*>(vals), n, s, sp);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(bps) * static_cast<unsigned>(t->sm_count);
-    return launch_k(t, kern, grid, block, 0, s, d, sp.keys, sp.vals, n, static_cast<uint64_t>(0), sp.counters, 512u);
+    e = launch_k(t, kern, grid, block, 0, s, d, sp.keys, sp.vals, n, static_cast<uint64_t>(0), sp.counters, 512u);
+    const cudaError_t r = scratch_release(t, s);
+    return e != cudaSuccess ? e : r;
   }
   if (op == WC_OP_COUNT || op == WC_OP_RETRIEVE) {
     auto kern = op == WC_OP_COUNT ? k_oa_walk<L, G, S, false> : k_oa_walk<L, G, S, true>;

@@ -120,7 +120,7 @@ cudaError_t run(const wc_table* t, const void* keys, const void* vals, uint64_t 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   sk<<<sg, kPartThreads, ssm, s>>>(static_cast<const Key*>(keys), static_cast<const Val*>(vals), n, m, hist, cursor,
-                                   pk, pv);
+                                   pk, pv, static_cast<uint2*>(nullptr));
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;  // no insert over a split that was never written
   const int block = lc.block_threads;

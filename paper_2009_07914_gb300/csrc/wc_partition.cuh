@@ -53,18 +53,6 @@ inline RegionMap region_map(const wc_table* t, int region_mib) {
   return m;
 }
 
-// Region of an output position: `per` consecutive positions per region.  Bit 31 of the
-// word carries a flag (the found bit of a retrieve result) and is not part of the
-// position.
-struct IndexMap {
-  uint32_t per;
-  uint32_t R;
-  __device__ __forceinline__ uint32_t of(uint32_t x) const {
-    const uint32_t r = (x & 0x7fffffffu) / per;
-    return r < R ? r : R - 1;
-  }
-};
-
 // Per-region counts of the batch (hist[R], zeroed by the caller).  Each warp keeps its
 // own shared-memory histogram, so atomics only collide inside a warp.
 constexpr int kHistWarps = kPartThreads / 32;
@@ -178,16 +166,19 @@ __device__ __forceinline__ void cp_async_elem(T* smem_dst, const T* gmem_src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Where the values of a split come from: read from `vals`, element i's input position i,
-// or 1 (vals is not read in the last two).
-enum { kValsRead = 0, kValsIota = 1, kValsOne = 2 };
+// Where the values of a split come from: read from `vals`, element i's position inside its
+// tile, or 1 (vals is not read in the last two).  With kValsLocal the split also leaves
+// runs[tile * R + r] = (start of the tile's run of region r in the output, its start in the
+// tile's own region order), from which k_unsplit puts results back in input order.
+enum { kValsRead = 0, kValsLocal = 1, kValsOne = 2 };
 
 template <class K, class V, class M = RegionMap, int kVals = kValsRead>
 __global__ void __launch_bounds__(kPartThreads) k_part_scatter(const K* __restrict__ keys, const V* __restrict__ vals,
                                                                uint64_t n, M m,
                                                                const unsigned int* __restrict__ hist,
                                                                unsigned long long* __restrict__ cursor,
-                                                               K* __restrict__ okeys, V* __restrict__ ovals) {
+                                                               K* __restrict__ okeys, V* __restrict__ ovals,
+                                                               uint2* __restrict__ runs) {
   extern __shared__ unsigned long long scatter_smem[];
   ScatterSmem<K, V>& S = *reinterpret_cast<ScatterSmem<K, V>*>(scatter_smem);
   constexpr bool kPre = scatter_prefetch<K, V>();
@@ -227,8 +218,8 @@ __global__ void __launch_bounds__(kPartThreads) k_part_scatter(const K* __restri
         } else {
           kk[k] = ldg_stream(keys + t0 + i);
         }
-        if constexpr (kVals == kValsIota) {
-          vv[k] = static_cast<V>(t0 + i);
+        if constexpr (kVals == kValsLocal) {
+          vv[k] = static_cast<V>(i);
         } else if constexpr (kVals == kValsOne) {
           vv[k] = V(1);
         } else if constexpr (kPre) {
@@ -246,8 +237,11 @@ __global__ void __launch_bounds__(kPartThreads) k_part_scatter(const K* __restri
       if (tile + gridDim.x < ntiles) prefetch(tile + gridDim.x);
     }
     block_scan_regions<unsigned int>(S.cnt, S.toff, m.R, S.w32);
-    for (uint32_t r = threadIdx.x; r < m.R; r += kPartThreads)
+    for (uint32_t r = threadIdx.x; r < m.R; r += kPartThreads) {
       if (S.cnt[r]) S.pos[r] = S.base[r] + atomicAdd(cursor + r, static_cast<unsigned long long>(S.cnt[r]));
+      if constexpr (kVals == kValsLocal)
+        runs[tile * m.R + r] = make_uint2(S.cnt[r] ? static_cast<uint32_t>(S.pos[r]) : 0u, S.toff[r]);
+    }
 #pragma unroll
     for (int k = 0; k < kPartItems; ++k) {
       if (rr[k] == 0xffffffffu) continue;
@@ -276,38 +270,36 @@ constexpr size_t scatter_smem_bytes() {
 
 // ---- host side -------------------------------------------------------------------------
 // A batch split by table region in the table's scratch buffer, plus kSplitCounters zeroed
-// chunk counters for the ordered sweeps of the kernels that consume it, and a zeroed
-// area for a second split (hist2 / cursor2) and `extra` bytes the caller asked for.
+// chunk counters for the ordered sweeps of the kernels that consume it, and `extra` bytes
+// the caller asked for.
 constexpr int kSplitCounters = 32;
-constexpr uint64_t kSplitHist = 0, kSplitCursor = 8192, kSplitCnt = 16384, kSplitHist2 = 16640,
-                   kSplitCursor2 = 20736, kSplitHeader = 29184;
-static_assert(kMaxRegions * sizeof(unsigned int) <= kSplitCursor2 - kSplitHist2, "hist2 area");
-static_assert(kMaxRegions * sizeof(unsigned long long) <= kSplitHeader - kSplitCursor2, "cursor2 area");
+constexpr uint64_t kSplitHist = 0, kSplitCursor = 8192, kSplitCnt = 16384, kSplitHeader = 16640;
+static_assert(kMaxRegions * sizeof(unsigned int) <= kSplitCursor - kSplitHist, "hist area");
+static_assert(kMaxRegions * sizeof(unsigned long long) <= kSplitCnt - kSplitCursor, "cursor area");
+static_assert(kSplitCounters * sizeof(unsigned long long) <= kSplitHeader - kSplitCnt, "counter area");
 
 template <class K, class V>
 struct RegionSplit {
   const K* keys;
   const V* vals;
   unsigned long long* counters;
-  unsigned int* hist2;          // second split: per-region counts (zeroed)
-  unsigned long long* cursor2;  // second split: per-region cursors (zeroed)
-  char* extra;                  // `extra` bytes, 256-byte aligned (not zeroed)
+  char* extra;  // `extra` bytes, 256-byte aligned (not zeroed)
 };
 
 inline uint64_t align256(uint64_t x) { return (x + 255) / 256 * 256; }
 
 // Regions of region_map(t, region_mib).  Scratch layout:
 // [header kSplitHeader B | keys | vals | extra], grown on demand.  kVals: where the values
-// come from (kValsIota: the input positions as uint32; kValsOne: all 1).
+// come from (kValsLocal: uint16 positions inside the tile, run starts to extra + runs_at;
+// kValsOne: all 1).  The caller hands the scratch on with scratch_release.
 template <class K, class V, int kVals = kValsRead>
 cudaError_t region_split(const wc_table* t, int region_mib, const K* keys, const V* vals, uint64_t n, cudaStream_t s,
-                         RegionSplit<K, V>& out, uint64_t extra = 0) {
-  static_assert(kMaxRegions * sizeof(unsigned long long) <= kSplitCnt - kSplitCursor, "cursor area");
+                         RegionSplit<K, V>& out, uint64_t extra = 0, uint64_t runs_at = 0) {
   const RegionMap m = region_map(t, region_mib);
   const uint64_t keys_off = kSplitHeader;
   const uint64_t vals_off = keys_off + align256(n * sizeof(K));
   const uint64_t extra_off = vals_off + align256(n * sizeof(V));
-  cudaError_t e = ensure_scratch(t, extra_off + extra, s);
+  cudaError_t e = ensure_scratch(t, extra_off + extra, s, lookup_scratch_likely(t, n));
   if (e != cudaSuccess) return e;
   char* sc = static_cast<char*>(t->d_scratch);
   auto* hist = reinterpret_cast<unsigned int*>(sc + kSplitHist);
@@ -332,13 +324,12 @@ cudaError_t region_split(const wc_table* t, int region_mib, const K* keys, const
   const unsigned sg = static_cast<unsigned>(
       std::min<uint64_t>(ntiles, static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count));
   hk<<<hg, kPartThreads, hsm, s>>>(keys, n, m, hist);
-  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, pk, pv);
+  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, pk, pv,
+                                   reinterpret_cast<uint2*>(sc + extra_off + runs_at));
   e = cudaGetLastError();
   out.keys = pk;
   out.vals = pv;
   out.counters = reinterpret_cast<unsigned long long*>(sc + kSplitCnt);
-  out.hist2 = reinterpret_cast<unsigned int*>(sc + kSplitHist2);
-  out.cursor2 = reinterpret_cast<unsigned long long*>(sc + kSplitCursor2);
   out.extra = sc + extra_off;
   return e;
 }

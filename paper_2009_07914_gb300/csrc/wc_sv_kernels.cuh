@@ -448,9 +448,10 @@ constexpr int retrieve_min_blocks() {
 template <class L, int G, int S, int H = 1>
 __global__ void __launch_bounds__(256, retrieve_min_blocks<L, S>()) k_sv_retrieve(TableDesc t, const typename L::Key* __restrict__ keys, uint64_t n,
                                                      uint64_t per_warp, typename L::Val* __restrict__ out,
-                                                     uint8_t* __restrict__ found) {
-  RangeSrc src(n, per_warp, nullptr, 0);
-  if (src.next >= src.end) return;
+                                                     uint8_t* __restrict__ found, unsigned long long* counter,
+                                                     uint32_t chunk) {
+  RangeSrc src(n, per_warp, counter, chunk);
+  if (counter == nullptr && src.next >= src.end) return;
   uint32_t flags = 0;
   EmitValue<L> emit{out, found, t.vals};
   sv_retrieve_range<L, G, S, EmitValue<L>, typename L::Key, false, H>(t, keys, src, emit, flags);
@@ -482,62 +483,6 @@ __global__ void __launch_bounds__(256) k_sv_retrieve_dedup(TableDesc t, const ty
   EmitValue<L> emit{out, found, t.vals};
   sv_retrieve_range<L, G, S, EmitValue<L>, typename L::Key, true, H>(t, keys, src, emit, flags);
   flush_flags(t.status, flags);
-}
-
-// Retrieve over a batch split by table region (the blocked scheme): warps pull chunks in
-// order, so the probes sweep the table region by region with the active regions in L2.
-// Results are written in the split order: rv[i] = value (or NOT_FOUND), rk[i] = the
-// query's input position qpos[i] with bit 31 set when found; a second split by position
-// and a placement pass put them back in input order.
-template <class L>
-struct EmitSwept {
-  const uint32_t* __restrict__ qpos;
-  uint32_t* __restrict__ rk;
-  typename L::Val* __restrict__ rv;
-  const void* vals;
-  __device__ void operator()(uint64_t i, bool hit, const typename L::Slot& s, uint64_t idx) const {
-    rv[i] = hit ? slot_value<L>(s, vals, idx) : L::kNotFound;
-    rk[i] = qpos[i] | (hit ? 0x80000000u : 0u);
-  }
-};
-
-template <class L, int G, int S, int H = 1>
-__global__ void __launch_bounds__(256) k_sv_retrieve_swept(TableDesc t, const typename L::Key* __restrict__ keys,
-                                                           const uint32_t* __restrict__ qpos, uint64_t n,
-                                                           unsigned long long* counter, uint32_t chunk,
-                                                           uint32_t* __restrict__ rk,
-                                                           typename L::Val* __restrict__ rv) {
-  RangeSrc src(n, 0, counter, chunk);
-  uint32_t flags = 0;
-  EmitSwept<L> emit{qpos, rk, rv, t.vals};
-  sv_retrieve_range<L, G, S, EmitSwept<L>, typename L::Key, false, H>(t, keys, src, emit, flags);
-  flush_flags(t.status, flags);
-}
-
-// Placement of split-ordered results: out[pos] = value, found[pos] = bit 31 of rk.  The
-// input is grouped by position region and the grid walks it front to back, so the
-// scattered stores of a moment fall into one or two L2-sized output regions.
-template <class V>
-__global__ void __launch_bounds__(256) k_place_results(const uint32_t* __restrict__ rk, const V* __restrict__ rv,
-                                                       uint64_t n, V* __restrict__ out, uint8_t* __restrict__ found) {
-  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint32_t k = ldg_stream(rk + i);
-    const V v = ldg_stream(rv + i);
-    const uint32_t pos = k & 0x7fffffffu;
-    out[pos] = v;
-    if (found) found[pos] = static_cast<uint8_t>(k >> 31);
-  }
-}
-
-// Exact per-region counts of the positions 0..n-1 (region r holds positions
-// [r * per, (r + 1) * per), the last one the rest).
-static __global__ void k_index_hist(unsigned int* __restrict__ hist, uint32_t R, uint32_t per, uint64_t n) {
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    const uint64_t lo = static_cast<uint64_t>(r) * per;
-    const uint64_t hi = r + 1 == R ? n : lo + per;
-    hist[r] = static_cast<unsigned int>(hi > lo ? hi - lo : 0);
-  }
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1,0 +1,129 @@
+"""Lookups one query per thread, and split by table region and put back: the sizes where the
+queue of a warp, a chunk of the sweep and a tile of the split begin and end, against the
+oracle's plain map; exact, integers.  Also what the split shares between calls: its scratch
+on two streams, and a lookup recorded into a CUDA graph."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import wc_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wc():
+    from paper_2009_07914_gb300 import build
+    build.build()
+    import paper_2009_07914_gb300 as m
+    return m
+
+
+def _inputs(kb, n, seed):
+    if kb == 4:
+        return wc_inputs.distinct_u32(seed, 2 * n), wc_inputs.uniform_u32(seed + 1, n)
+    return wc_inputs.distinct_u64(seed, 2 * n), wc_inputs.uniform_u64(seed + 1, n)
+
+
+def _device(torch, a):
+    return torch.from_numpy(a.view(np.int32 if a.itemsize == 4 else np.int64)).cuda()
+
+
+@pytest.mark.parametrize("blocked", [False, True], ids=["direct", "split"])
+@pytest.mark.parametrize("kb,W,soa,bits", [(4, 8, 0, 1), (4, 4, 0, 0), (8, 4, 0, 1), (8, 2, 0, 0), (4, 16, 1, 0),
+                                           (8, 8, 1, 0), (4, 16, 0, 0)])
+def test_batch_edges(wc, kb, W, soa, bits, blocked):
+    import torch
+    from paper_2009_07914_gb300 import api
+    n = 30_011
+    keys, vals = _inputs(kb, n, 0x10C + kb + W)
+    opt = (wc.WC_OPT_SOA if soa else 0) | (wc.WC_OPT_OVERFLOW_BITS if bits else 0)
+    t = wc.SingleValueTable(kb, kb, min_capacity=int(n / 0.97) + 1, window_width=W, options=opt)
+    o = oracle.SingleValue(kb, kb)
+    t.insert(keys[:n], vals)
+    o.insert(keys[:n], vals)
+    if blocked:
+        lc = api.wc_table_get_launch(t.handle, wc.WC_OP_RETRIEVE)
+        t.set_launch(wc.WC_OP_RETRIEVE, lc["group_size"], scheme=wc.WC_SCHEME_BLOCKED, region_mib=1)
+    q = keys[wc_inputs.shuffle_index(9, 2 * n)]
+    q[5::97] = 0
+    q[6::97] = 2 ** (8 * kb) - 1
+    q[7::97] = keys[0]  # the same query again and again
+    for m in (1, 31, 32, 33, 511, 512, 513, 4095, 4096, 4097, 2 * n):
+        for off in (0, 1):  # outputs off their natural start
+            qd = _device(torch, np.concatenate([q[:1], q[:m]]))[1:]
+            out = torch.full((m + 3,), 77, dtype=qd.dtype, device="cuda")
+            found = torch.full((m + 3,), 9, dtype=torch.uint8, device="cuda")
+            api.wc_retrieve(t.handle, qd, out[off:off + m], found[off:off + m])
+            eo, ef, _ = o.retrieve(q[:m])
+            np.testing.assert_array_equal(out[off:off + m].cpu().numpy().view(eo.dtype), eo)
+            np.testing.assert_array_equal(found[off:off + m].cpu().numpy(), ef)
+            assert (out[off + m:] == 77).all() and (found[off + m:] == 9).all()
+            api.wc_contains(t.handle, qd, found[off:off + m])
+            np.testing.assert_array_equal(found[off:off + m].cpu().numpy(), ef)
+
+
+def test_split_scratch_is_shared_in_order_between_streams(wc):
+    import torch
+    from paper_2009_07914_gb300 import api
+    n = 400_003
+    keys, vals = _inputs(4, n, 0x5C2)
+    t = wc.SingleValueTable(4, 4, min_capacity=int(n / 0.9) + 1)
+    t.insert(keys[:n], vals)
+    lc = api.wc_table_get_launch(t.handle, wc.WC_OP_RETRIEVE)
+    t.set_launch(wc.WC_OP_RETRIEVE, lc["group_size"], scheme=wc.WC_SCHEME_BLOCKED, region_mib=1)
+    o = oracle.SingleValue(4, 4)
+    o.insert(keys[:n], vals)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    work = []
+    for i in range(12):  # batches of several sizes: the scratch grows between streams
+        q = keys[wc_inputs.shuffle_index(i, 2 * n)][:20_000 + 60_000 * (i % 5)]
+        work.append((q, _device(torch, q), torch.empty(q.size, dtype=torch.int32, device="cuda"),
+                     torch.empty(q.size, dtype=torch.uint8, device="cuda")))
+    torch.cuda.synchronize()
+    for i, (q, qd, out, found) in enumerate(work):
+        api.wc_retrieve(t.handle, qd, out, found, stream=streams[i % 3])
+    torch.cuda.synchronize()
+    for q, _, out, found in work:
+        eo, ef, _ = o.retrieve(q)
+        np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), eo)
+        np.testing.assert_array_equal(found.cpu().numpy(), ef)
+
+
+def test_lookup_in_a_graph_keeps_no_scratch(wc):
+    """A batch that is split outside a capture (a table above 512 MiB) is recorded in input
+    order: the graph holds no buffer of the table, and replays after the scratch has moved."""
+    import torch
+    from paper_2009_07914_gb300 import api
+    slots = 70_000_000
+    n = 1_000_003
+    keys, vals = _inputs(4, n, 0x6AF)
+    t = wc.SingleValueTable(4, 4, min_capacity=slots, window_width=8)
+    assert t.info["table_bytes"] > 512 << 20
+    t.insert(keys[:n], vals)
+    m = t.info["table_bytes"] // 64 + 1
+    q = np.resize(keys, m)
+    qd = _device(torch, q)
+    out, found = torch.empty(m, dtype=torch.int32, device="cuda"), torch.empty(m, dtype=torch.uint8, device="cuda")
+    before = api.wc_table_get_info(t.handle)["work_bytes"]
+    api.wc_contains(t.handle, qd[:64], found[:64])  # the kernel is loaded before the capture
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        api.wc_retrieve(t.handle, qd, out, found, stream=s)
+    assert api.wc_table_get_info(t.handle)["work_bytes"] == before
+    api.wc_retrieve(t.handle, qd, out, found)
+    assert api.wc_table_get_info(t.handle)["work_bytes"] > before  # the same call outside is split
+    torch.cuda.synchronize()
+    eo, ef = np.resize(np.concatenate([vals, np.full(n, 2 ** 32 - 1, np.uint32)]), m), np.resize(
+        np.repeat(np.array([1, 0], np.uint8), n), m)
+    for again in (False, True):
+        if again:
+            out.fill_(5)
+            found.fill_(5)
+            g.replay()
+            torch.cuda.synchronize()
+        np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), eo)
+        np.testing.assert_array_equal(found.cpu().numpy(), ef)
