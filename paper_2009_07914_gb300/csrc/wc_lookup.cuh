@@ -355,11 +355,12 @@ struct QuerySplit {
 template <class K, class V>
 cudaError_t query_split(const wc_table* t, int region_mib, const K* keys, uint64_t n, cudaStream_t s,
                         QuerySplit<K, V>& q) {
-  q.R = region_map(t, region_mib).R;
+  const RegionMap m = region_map(t, region_mib);
+  q.R = m.R;
   const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
   const uint64_t rv_bytes = align256(n * sizeof(V)), rf_bytes = align256(n);
   const uint64_t runs_bytes = ntiles * q.R * sizeof(uint2);
-  const cudaError_t e = region_split<K, uint16_t, kValsLocal>(t, region_mib, keys, nullptr, n, s, q.sp,
+  const cudaError_t e = region_split<K, uint16_t, kValsLocal>(t, m, keys, nullptr, n, s, q.sp,
                                                               rv_bytes + rf_bytes + runs_bytes, rv_bytes + rf_bytes);
   if (e != cudaSuccess) return e;
   q.rv = reinterpret_cast<V*>(q.sp.extra);

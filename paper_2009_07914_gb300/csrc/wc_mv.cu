@@ -39,7 +39,7 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
   cudaError_t e = cudaSuccess;
   if (n >= (1ull << 20) && t->table_bytes > (64ull << 20)) {
     RegionSplit<KIn, V> sp;
-    e = region_split(t, 32, k, static_cast<const V*>(vals), n, s, sp, rec_bytes);
+    e = region_split(t, region_map(t, 32), k, static_cast<const V*>(vals), n, s, sp, rec_bytes);
     if (e != cudaSuccess) return e;
     k = sp.keys;
     vals = sp.vals;

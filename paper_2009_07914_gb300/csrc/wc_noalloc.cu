@@ -29,7 +29,7 @@
 namespace wc {
 namespace {
 
-constexpr uint64_t kHeadBytes = 64ull << 10;  // hist (4 KiB) | cursors (8 KiB) | work counter
+constexpr uint64_t kHeadBytes = 64ull << 10;  // hist (8 KiB) | cursors (8 KiB) | work counter
 constexpr uint64_t kCursorOff = 8192, kWorkOff = 16384;
 constexpr uint64_t kScratchBytes = kHeadBytes + WC_NOALLOC_SCRATCH_BYTES;
 constexpr int kMaxDevices = 64;
@@ -97,31 +97,15 @@ cudaError_t run(const wc_table* t, const void* keys, const void* vals, uint64_t 
   const wc_launch& lc = t->launch[WC_OP_INSERT];
   const RegionMap m = region_map(t, lc.region_mib);
   auto* hist = reinterpret_cast<unsigned int*>(sc);
-  auto* cursor = reinterpret_cast<unsigned long long*>(sc + kCursorOff);
+  auto* cursor = reinterpret_cast<unsigned int*>(sc + kCursorOff);
   auto* work = reinterpret_cast<unsigned long long*>(sc + kWorkOff);
   Key* pk = reinterpret_cast<Key*>(sc + kHeadBytes);
   Val* pv = reinterpret_cast<Val*>(sc + kHeadBytes + (n * sizeof(Key) + 255) / 256 * 256);
   cudaError_t e = cudaMemsetAsync(sc, 0, kWorkOff + 8, s);
   if (e != cudaSuccess) return e;
-  auto hk = k_part_hist<Key>;
-  auto sk = k_part_scatter<Key, Val>;
   auto ik = k_sv_insert<L, G, S, H>;
-  const size_t hsm = static_cast<size_t>(kHistWarps) * m.R * sizeof(unsigned int);
-  const size_t ssm = scatter_smem_bytes<Key, Val>();
-  e = cudaFuncSetAttribute(hk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kHistWarps * kMaxRegions * 4));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ssm));
-  if (e != cudaSuccess) return e;
-  const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
-  const unsigned hg = static_cast<unsigned>(std::min<uint64_t>(
-      (n + kPartTile - 1) / kPartTile, static_cast<uint64_t>(occupancy_smem(hk, kPartThreads, hsm)) * t->sm_count));
-  const unsigned sg = static_cast<unsigned>(
-      std::min<uint64_t>(ntiles, static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count));
-  hk<<<hg, kPartThreads, hsm, s>>>(static_cast<const Key*>(keys), n, m, hist);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  sk<<<sg, kPartThreads, ssm, s>>>(static_cast<const Key*>(keys), static_cast<const Val*>(vals), n, m, hist, cursor,
-                                   pk, pv, static_cast<uint2*>(nullptr));
-  e = cudaGetLastError();
+  e = split_launch<Key, Val>(t, m, static_cast<const Key*>(keys), static_cast<const Val*>(vals), n, hist, cursor, pk,
+                             pv, nullptr, s);
   if (e != cudaSuccess) return e;  // no insert over a split that was never written
   const int block = lc.block_threads;
   const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : occupancy(ik, block);

@@ -10,6 +10,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "wc_device.cuh"
 #include "wc_internal.h"
@@ -20,7 +21,8 @@ namespace wc {
 constexpr int kPartThreads = 512;
 constexpr int kPartItems = 8;
 constexpr int kPartTile = kPartThreads * kPartItems;
-constexpr int kMaxRegions = 1024;
+constexpr int kMaxRegions = 1024;      // of a sweep (region_map)
+constexpr int kMaxSplitRegions = 2048; // of any split (header areas)
 
 struct RegionMap {
   uint64_t seed;
@@ -31,8 +33,7 @@ struct RegionMap {
   __device__ __forceinline__ uint32_t of(K key) const {
     uint32_t w, step;
     probe_init(static_cast<uint64_t>(key), seed, p, w, step);
-    const uint32_t r = w >> shift;
-    return r < R ? r : R - 1;
+    return w >> shift;  // below R = ceil(p / 2^shift), since w < p
   }
 };
 
@@ -53,17 +54,19 @@ inline RegionMap region_map(const wc_table* t, int region_mib) {
   return m;
 }
 
-// Per-region counts of the batch (hist[R], zeroed by the caller).  Each warp keeps its
-// own shared-memory histogram, so atomics only collide inside a warp.
+// Per-region counts of the batch (hist[R], zeroed by the caller).  Warps share `copies`
+// shared-memory histograms (one each while the regions are few), so few atomics collide.
 constexpr int kHistWarps = kPartThreads / 32;
+
+inline uint32_t hist_copies(uint32_t R) { return R <= 512 ? kHistWarps : R <= 1024 ? 8 : 4; }
 
 template <class K>
 __global__ void __launch_bounds__(kPartThreads) k_part_hist(const K* __restrict__ keys, uint64_t n, RegionMap m,
-                                                            unsigned int* __restrict__ hist) {
-  extern __shared__ unsigned int s_hw[];  // kHistWarps * R
-  for (uint32_t i = threadIdx.x; i < kHistWarps * m.R; i += kPartThreads) s_hw[i] = 0;
+                                                            unsigned int* __restrict__ hist, uint32_t copies) {
+  extern __shared__ unsigned int s_hw[];  // copies * R
+  for (uint32_t i = threadIdx.x; i < copies * m.R; i += kPartThreads) s_hw[i] = 0;
   __syncthreads();
-  unsigned int* mine = s_hw + (threadIdx.x >> 5) * m.R;
+  unsigned int* mine = s_hw + ((threadIdx.x >> 5) & (copies - 1)) * m.R;
   // kPartItems independent loads in flight per thread (block b takes elements
   // [b * kPartTile, (b + 1) * kPartTile) of every grid-wide stride, one per thread per item)
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kPartTile;
@@ -81,77 +84,63 @@ __global__ void __launch_bounds__(kPartThreads) k_part_hist(const K* __restrict_
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) {
     unsigned int c = 0;
-#pragma unroll
-    for (int w = 0; w < kHistWarps; ++w) c += s_hw[w * m.R + i];
+    for (uint32_t w = 0; w < copies; ++w) c += s_hw[w * m.R + i];
     if (c) atomicAdd(hist + i, c);
   }
 }
 
-// Exclusive scan of cnt[0..R) into off[0..R) by the whole block (R <= kMaxRegions);
-// returns the total.  Every thread handles kMaxRegions / kPartThreads consecutive entries.
-template <class T>
-__device__ __forceinline__ T block_scan_regions(const T* cnt, T* off, uint32_t R, T* s_w) {
-  constexpr int kPer = kMaxRegions / kPartThreads;
+// Exclusive scan of cnt[0..R) by the whole block (R <= kMaxSplitRegions): give(r, before,
+// cnt[r]) is called once per region; ends with a barrier.  Up to 256 regions are scanned by
+// the first warp alone, 32 at a time, while the others wait (fewer instructions than every
+// warp's part of a block-wide scan).
+template <class Give>
+__device__ __forceinline__ void scan_regions(const uint32_t* cnt, uint32_t R, uint32_t* s_w, Give give) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (R <= 256) {
+    if (warp == 0) {
+      uint32_t run = 0;
+      for (uint32_t r0 = 0; r0 < R; r0 += 32) {
+        const uint32_t c = r0 + lane < R ? cnt[r0 + lane] : 0u;
+        uint32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(kFull, inc, o);
+          if (lane >= o) inc += y;
+        }
+        if (r0 + lane < R) give(r0 + lane, run + inc - c, c);
+        run += __shfl_sync(kFull, inc, 31);
+      }
+    }
+    __syncthreads();
+    return;
+  }
+  constexpr int kPer = kMaxSplitRegions / kPartThreads;
   const uint32_t b0 = threadIdx.x * kPer;
-  T v[kPer];
-  T sum = 0;
+  uint32_t v[kPer], sum = 0;
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
-    v[k] = b0 + k < R ? cnt[b0 + k] : T(0);
+    v[k] = b0 + k < R ? cnt[b0 + k] : 0u;
     sum += v[k];
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T inc = sum;
+  uint32_t inc = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const T y = __shfl_up_sync(kFull, inc, o);
+    const uint32_t y = __shfl_up_sync(kFull, inc, o);
     if (lane >= o) inc += y;
   }
   if (lane == 31) s_w[warp] = inc;
   __syncthreads();
-  T before = 0, total = 0;
+  uint32_t run = inc - sum;
 #pragma unroll
-  for (int w = 0; w < kPartThreads / 32; ++w) {
-    if (w < warp) before += s_w[w];
-    total += s_w[w];
-  }
-  T run = before + inc - sum;
+  for (int w = 0; w < kPartThreads / 32; ++w)
+    if (w < warp) run += s_w[w];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
-    if (b0 + k < R) off[b0 + k] = run;
+    if (b0 + k < R) give(b0 + k, run, v[k]);
     run += v[k];
   }
   __syncthreads();
-  return total;
 }
-
-// Scatter (keys, vals) into region order.  Per tile: rank every element inside its
-// region with shared-memory atomics, reserve one run per region in the output with one
-// global atomic on cursor[r] (zeroed by the caller), stage the tile in shared memory
-// grouped by region, then copy the runs out with consecutive threads on consecutive
-// addresses.  For pairs of at most 8 bytes the next tile's input is copied into shared
-// memory with cp.async while the current tile is ranked and written out, so the input
-// stream never stops (wider pairs would halve the resident blocks and read directly).
-template <class K, class V>
-constexpr bool scatter_prefetch() {
-  return sizeof(K) + sizeof(V) <= 8;
-}
-
-template <class K, class V>
-struct ScatterSmem {
-  static constexpr int kIn = scatter_prefetch<K, V>() ? kPartTile : 1;
-  K keys[kPartTile];
-  V vals[kPartTile];
-  unsigned short reg[kPartTile];
-  unsigned int cnt[kMaxRegions];
-  unsigned int toff[kMaxRegions];
-  unsigned long long base[kMaxRegions];
-  unsigned long long pos[kMaxRegions];
-  unsigned long long w64[kPartThreads / 32];
-  unsigned int w32[kPartThreads / 32];
-  K in_keys[kIn];  // the next tile's input (prefetching layouts only)
-  V in_vals[kIn];
-};
 
 // Asynchronous global -> shared copy of one 4- or 8-byte element (cp.async, L1 bypassed
 // for the streamed input with an evict-first L2 policy), and the wait for all of them.
@@ -167,105 +156,158 @@ __device__ __forceinline__ void cp_async_elem(T* smem_dst, const T* gmem_src) {
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Where the values of a split come from: read from `vals`, element i's position inside its
-// tile, or 1 (vals is not read in the last two).  With kValsLocal the split also leaves
-// runs[tile * R + r] = (start of the tile's run of region r in the output, its start in the
-// tile's own region order), from which k_unsplit puts results back in input order.
-enum { kValsRead = 0, kValsLocal = 1, kValsOne = 2 };
+// tile, or there are none (vals is read in the first only, ovals not written in the last).
+// With kValsLocal the split also leaves runs[tile * R + r] = (start of the tile's run of
+// region r in the output, its start in the tile's own region order), from which k_unsplit
+// puts results back in input order.
+enum { kValsRead = 0, kValsLocal = 1, kValsNone = 2 };
 
-template <class K, class V, class M = RegionMap, int kVals = kValsRead>
-__global__ void __launch_bounds__(kPartThreads) k_part_scatter(const K* __restrict__ keys, const V* __restrict__ vals,
-                                                               uint64_t n, M m,
-                                                               const unsigned int* __restrict__ hist,
-                                                               unsigned long long* __restrict__ cursor,
-                                                               K* __restrict__ okeys, V* __restrict__ ovals,
-                                                               uint2* __restrict__ runs) {
+// Scatter (keys, vals) into region order.  Per tile: rank every element inside its region
+// with shared-memory atomics, reserve one run per region in the output with one global
+// atomic on cursor[r] (zeroed by the caller), stage the tile in shared memory grouped by
+// region, then copy the runs out with consecutive threads on consecutive addresses.
+// Issue and the shared-memory pipe bound it (both about two thirds busy), so what an
+// element takes is kept short: its place in the output is delta[region] + its place in the
+// staged tile, position and region of a split with positions share one staged word, and the
+// scan over the regions is one warp's.  Pairs of at most 8 bytes come through a buffer that
+// cp.async fills for the next tile while this one is written out (no input is held in
+// registers, so three blocks fit an SM); wider ones are read into registers, two blocks.
+// One GB300, before -> now: 2^28 pairs of 8+4 bytes 1.94 -> 1.39 ms, 8+8 2.45 -> 2.17;
+// 2^27 queries of 4 bytes (with positions) 0.59 -> 0.49, 2^27 4+4-byte pairs 0.65 -> 0.66
+// (3.2 TB/s); 60 M keys alone 0.26 -> 0.19 (a set's 4-byte values of 1 are not written).
+template <class K, class V, int kVals>
+struct SplitTile {
+  static constexpr bool kPre = sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) <= 8 && sizeof(K) == 4;
+  static constexpr int kMinBlocks = kPre ? 3 : 2;
+  // shared bytes of one element: staged key, value and region, input buffer
+  static constexpr size_t kElem = sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) + (kVals == kValsLocal ? 4 : 2) +
+                                  (kPre ? sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) : 0);
+  static constexpr size_t smem_bytes(uint32_t R, int tile) {
+    return kElem * tile + 4 * (4ull * R + kPartThreads / 32);
+  }
+};
+
+template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
+__global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlocks))
+    k_part_scatter(const K* __restrict__ keys, const V* __restrict__ vals, uint64_t n, RegionMap m,
+                   const unsigned int* __restrict__ hist, unsigned int* __restrict__ cursor, K* __restrict__ okeys,
+                   V* __restrict__ ovals, uint2* __restrict__ runs) {
+  using Tile = SplitTile<K, V, kVals>;
+  constexpr bool kPre = Tile::kPre, kRead = kVals == kValsRead;
+  constexpr int kTile = kPartThreads * kItems;
   extern __shared__ unsigned long long scatter_smem[];
-  ScatterSmem<K, V>& S = *reinterpret_cast<ScatterSmem<K, V>*>(scatter_smem);
-  constexpr bool kPre = scatter_prefetch<K, V>();
-  const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
-  // copy tile `tl`'s input into S.in_keys / S.in_vals (prefetching layouts)
-  auto prefetch = [&](uint64_t tl) {
-    const uint64_t b = tl * kPartTile;
-    const uint32_t cnt = static_cast<uint32_t>(n - b < kPartTile ? n - b : kPartTile);
+  char* at = reinterpret_cast<char*>(scatter_smem);
+  auto carve = [&](size_t bytes) {
+    char* p = at;
+    at += bytes;
+    return p;
+  };
+  // 4+4-byte pairs are staged together (one store and one load of 8 bytes)
+  constexpr bool kPair = kRead && sizeof(K) == 4 && sizeof(V) == 4;
+  uint2* s_pair = reinterpret_cast<uint2*>(at);
+  K* s_key = reinterpret_cast<K*>(carve(sizeof(K) * kTile));
+  V* s_val = reinterpret_cast<V*>(carve(kRead ? sizeof(V) * kTile : 0));
+  K* in_key = reinterpret_cast<K*>(carve(kPre ? sizeof(K) * kTile : 0));
+  V* in_val = reinterpret_cast<V*>(carve(kPre && kRead ? sizeof(V) * kTile : 0));
+  using Reg = typename std::conditional<kVals == kValsLocal, uint32_t, uint16_t>::type;
+  Reg* s_reg = reinterpret_cast<Reg*>(carve(sizeof(Reg) * kTile));  // region (<< 16 | position, with kValsLocal)
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(carve(4ull * m.R));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(carve(4ull * m.R));    // start in the staged tile
+  uint32_t* s_delta = reinterpret_cast<uint32_t*>(carve(4ull * m.R));  // output place - staged place
+  uint32_t* s_base = reinterpret_cast<uint32_t*>(carve(4ull * m.R));   // the region's start in the output
+  uint32_t* s_w = reinterpret_cast<uint32_t*>(carve(4ull * (kPartThreads / 32)));
+  const uint32_t nn = static_cast<uint32_t>(n);  // n < 2^32: places and counts are 32 bits
+  const uint32_t ntiles = static_cast<uint32_t>((n + kTile - 1) / kTile);
+  // copy tile `tl`'s input into the input buffer
+  auto prefetch = [&](uint32_t tl) {
+    const uint32_t b = tl * kTile;
+    const uint32_t cnt = nn - b < kTile ? nn - b : kTile;
     for (uint32_t i = threadIdx.x; i < cnt; i += kPartThreads) {
-      cp_async_elem(S.in_keys + i, keys + b + i);
-      if constexpr (kVals == kValsRead) cp_async_elem(S.in_vals + i, vals + b + i);
+      cp_async_elem(in_key + i, keys + b + i);
+      if constexpr (kRead) cp_async_elem(in_val + i, vals + b + i);
     }
   };
   if constexpr (kPre) {
     if (blockIdx.x < ntiles) prefetch(blockIdx.x);
   }
   // region bases: exclusive prefix of the histogram (every block recomputes it)
-  for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) S.pos[i] = hist[i];
+  for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) s_cnt[i] = hist[i];
   __syncthreads();
-  block_scan_regions<unsigned long long>(S.pos, S.base, m.R, S.w64);
-  for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) S.cnt[i] = 0;
+  scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t) { s_base[r] = before; });
+  for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) s_cnt[i] = 0;
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const uint32_t t0 = tile * kTile;
+    const uint32_t tn = nn - t0 < kTile ? nn - t0 : kTile;
     if constexpr (kPre) cp_async_wait_all();  // this tile's input is in shared memory
     __syncthreads();
-    const uint64_t t0 = tile * kPartTile;
-    const uint32_t tn = static_cast<uint32_t>(n - t0 < kPartTile ? n - t0 : kPartTile);
-    K kk[kPartItems];
-    V vv[kPartItems];
-    uint32_t rr[kPartItems], rank[kPartItems];
+    K kk[kPre ? 1 : kItems];
+    V vv[kPre || !kRead ? 1 : kItems];
+    uint32_t rr[kItems];  // region << 16 | rank (a tile holds fewer than 2^16 elements)
+    if constexpr (!kPre) {
 #pragma unroll
-    for (int k = 0; k < kPartItems; ++k) {
+      for (int k = 0; k < kItems; ++k) {
+        const uint32_t i = k * kPartThreads + threadIdx.x;
+        kk[k] = i < tn ? ldg_stream(keys + t0 + i) : K(0);
+        if constexpr (kRead) vv[k] = i < tn ? ldg_stream(vals + t0 + i) : V(0);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
       const uint32_t i = k * kPartThreads + threadIdx.x;
-      rr[k] = 0xffffffffu;
       if (i < tn) {
-        if constexpr (kPre) {
-          kk[k] = S.in_keys[i];
-        } else {
-          kk[k] = ldg_stream(keys + t0 + i);
-        }
-        if constexpr (kVals == kValsLocal) {
-          vv[k] = static_cast<V>(i);
-        } else if constexpr (kVals == kValsOne) {
-          vv[k] = V(1);
-        } else if constexpr (kPre) {
-          vv[k] = S.in_vals[i];
-        } else {
-          vv[k] = ldg_stream(vals + t0 + i);
-        }
-        rr[k] = m.of(kk[k]);
-        rank[k] = atomicAdd(S.cnt + rr[k], 1u);
+        uint32_t r;
+        if constexpr (kPre) r = m.of(in_key[i]);
+        else r = m.of(kk[k]);
+        rr[k] = r << 16 | atomicAdd(s_cnt + r, 1u);
       }
     }
     __syncthreads();
-    // the input buffer is free again: start copying the block's next tile
-    if constexpr (kPre) {
-      if (tile + gridDim.x < ntiles) prefetch(tile + gridDim.x);
-    }
-    block_scan_regions<unsigned int>(S.cnt, S.toff, m.R, S.w32);
-    for (uint32_t r = threadIdx.x; r < m.R; r += kPartThreads) {
-      if (S.cnt[r]) S.pos[r] = S.base[r] + atomicAdd(cursor + r, static_cast<unsigned long long>(S.cnt[r]));
-      if constexpr (kVals == kValsLocal)
-        runs[tile * m.R + r] = make_uint2(S.cnt[r] ? static_cast<uint32_t>(S.pos[r]) : 0u, S.toff[r]);
-    }
+    scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t c) {
+      const uint32_t p = c ? s_base[r] + atomicAdd(cursor + r, c) : 0u;
+      s_off[r] = before;
+      s_delta[r] = p - before;
+      if constexpr (kVals == kValsLocal) runs[static_cast<uint64_t>(tile) * m.R + r] = make_uint2(p, before);
+    });
 #pragma unroll
-    for (int k = 0; k < kPartItems; ++k) {
-      if (rr[k] == 0xffffffffu) continue;
-      const uint32_t o = S.toff[rr[k]] + rank[k];
-      S.keys[o] = kk[k];
-      S.vals[o] = vv[k];
-      S.reg[o] = static_cast<unsigned short>(rr[k]);
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < tn; i += kPartThreads) {
-      const uint32_t r = S.reg[i];
-      const uint64_t o = S.pos[r] + (i - S.toff[r]);
-      if (o < n) {  // always true when hist holds this batch's counts
-        okeys[o] = S.keys[i];
-        ovals[o] = S.vals[i];
+    for (int k = 0; k < kItems; ++k) {
+      const uint32_t i = k * kPartThreads + threadIdx.x;
+      if (i < tn) {
+        const uint32_t r = rr[k] >> 16, o = s_off[r] + (rr[k] & 0xffffu);
+        if constexpr (kPair) {
+          s_pair[o] = make_uint2(in_key[i], in_val[i]);
+        } else {
+          if constexpr (kPre) s_key[o] = in_key[i];
+          else s_key[o] = kk[k];
+          if constexpr (kRead) s_val[o] = vv[k];
+        }
+        if constexpr (kVals == kValsLocal) s_reg[o] = r << 16 | i;
+        else s_reg[o] = static_cast<Reg>(r);
       }
     }
     __syncthreads();
+    // the input buffer and the counters are free again
+    if constexpr (kPre) {
+      if (ntiles - tile > gridDim.x) prefetch(tile + gridDim.x);
+    }
+    for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) s_cnt[i] = 0;
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < tn; i += kPartThreads) {
+      const uint32_t x = s_reg[i];
+      const uint32_t o = s_delta[kVals == kValsLocal ? x >> 16 : x] + i;
+      if (o < nn) {  // always true when hist holds this batch's counts
+        if constexpr (kPair) {
+          const uint2 p = s_pair[i];
+          okeys[o] = p.x;
+          ovals[o] = p.y;
+        } else {
+          okeys[o] = s_key[i];
+          if constexpr (kVals == kValsLocal) ovals[o] = static_cast<V>(x & 0xffffu);
+          else if constexpr (kRead) ovals[o] = s_val[i];
+        }
+      }
+    }
   }
-}
-
-template <class K, class V>
-constexpr size_t scatter_smem_bytes() {
-  return sizeof(ScatterSmem<K, V>);
+  if constexpr (kPre) cp_async_wait_all();
 }
 
 // ---- host side -------------------------------------------------------------------------
@@ -274,64 +316,73 @@ constexpr size_t scatter_smem_bytes() {
 // the caller asked for.
 constexpr int kSplitCounters = 32;
 constexpr uint64_t kSplitHist = 0, kSplitCursor = 8192, kSplitCnt = 16384, kSplitHeader = 16640;
-static_assert(kMaxRegions * sizeof(unsigned int) <= kSplitCursor - kSplitHist, "hist area");
-static_assert(kMaxRegions * sizeof(unsigned long long) <= kSplitCnt - kSplitCursor, "cursor area");
+static_assert(kMaxSplitRegions * sizeof(unsigned int) <= kSplitCursor - kSplitHist, "hist area");
+static_assert(kMaxSplitRegions * sizeof(unsigned int) <= kSplitCnt - kSplitCursor, "cursor area");
 static_assert(kSplitCounters * sizeof(unsigned long long) <= kSplitHeader - kSplitCnt, "counter area");
 
 template <class K, class V>
 struct RegionSplit {
   const K* keys;
   const V* vals;
+  const unsigned int* hist;  // keys of every region
   unsigned long long* counters;
   char* extra;  // `extra` bytes, 256-byte aligned (not zeroed)
 };
 
 inline uint64_t align256(uint64_t x) { return (x + 255) / 256 * 256; }
 
-// Regions of region_map(t, region_mib).  Scratch layout:
-// [header kSplitHeader B | keys | vals | extra], grown on demand.  kVals: where the values
-// come from (kValsLocal: uint16 positions inside the tile, run starts to extra + runs_at;
-// kValsOne: all 1).  The caller hands the scratch on with scratch_release.
-template <class K, class V, int kVals = kValsRead>
-cudaError_t region_split(const wc_table* t, int region_mib, const K* keys, const V* vals, uint64_t n, cudaStream_t s,
-                         RegionSplit<K, V>& out, uint64_t extra = 0, uint64_t runs_at = 0) {
-  const RegionMap m = region_map(t, region_mib);
+// The two kernels of a split: hist and cursor are m.R zeroed words each.
+template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
+cudaError_t split_launch(const wc_table* t, const RegionMap& m, const K* keys, const V* vals, uint64_t n,
+                         unsigned int* hist, unsigned int* cursor, K* okeys, V* ovals, uint2* runs, cudaStream_t s) {
+  auto hk = k_part_hist<K>;
+  auto sk = k_part_scatter<K, V, kVals, kItems>;
+  using Tile = SplitTile<K, V, kVals>;
+  constexpr int kTile = kPartThreads * kItems;
+  const uint32_t copies = hist_copies(m.R);
+  const size_t hsm = static_cast<size_t>(copies) * m.R * sizeof(unsigned int);
+  const size_t ssm = Tile::smem_bytes(m.R, kTile);
+  static const cudaError_t attr = [&] {
+    const cudaError_t e = cudaFuncSetAttribute(hk, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistWarps * 512 * 4);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(Tile::smem_bytes(kMaxSplitRegions, kTile)));
+  }();
+  if (attr != cudaSuccess) return attr;
+  const uint64_t hist_most = static_cast<uint64_t>(occupancy_smem(hk, kPartThreads, hsm)) * t->sm_count;
+  const uint64_t split_most = static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count;
+  const unsigned hg = static_cast<unsigned>(std::min<uint64_t>((n + kPartTile - 1) / kPartTile, hist_most));
+  const unsigned sg = static_cast<unsigned>(std::min<uint64_t>((n + kTile - 1) / kTile, split_most));
+  hk<<<hg, kPartThreads, hsm, s>>>(keys, n, m, hist, copies);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;  // no split without its counts
+  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, okeys, ovals, runs);
+  return cudaGetLastError();
+}
+
+// Regions of m.  Scratch layout: [header kSplitHeader B | keys | vals | extra], grown on
+// demand.  kVals: where the values come from (kValsLocal: uint16 positions inside the tile,
+// run starts to extra + runs_at).  The caller hands the scratch on with scratch_release.
+template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
+cudaError_t region_split(const wc_table* t, const RegionMap& m, const K* keys, const V* vals, uint64_t n,
+                         cudaStream_t s, RegionSplit<K, V>& out, uint64_t extra = 0, uint64_t runs_at = 0) {
   const uint64_t keys_off = kSplitHeader;
   const uint64_t vals_off = keys_off + align256(n * sizeof(K));
-  const uint64_t extra_off = vals_off + align256(n * sizeof(V));
+  const uint64_t extra_off = vals_off + (kVals == kValsNone ? 0 : align256(n * sizeof(V)));
   cudaError_t e = ensure_scratch(t, extra_off + extra, s, lookup_scratch_likely(t, n));
   if (e != cudaSuccess) return e;
   char* sc = static_cast<char*>(t->d_scratch);
+  out.keys = reinterpret_cast<K*>(sc + keys_off);
+  out.vals = kVals == kValsNone ? nullptr : reinterpret_cast<V*>(sc + vals_off);
   auto* hist = reinterpret_cast<unsigned int*>(sc + kSplitHist);
-  auto* cursor = reinterpret_cast<unsigned long long*>(sc + kSplitCursor);
-  K* pk = reinterpret_cast<K*>(sc + keys_off);
-  V* pv = reinterpret_cast<V*>(sc + vals_off);
-  e = cudaMemsetAsync(sc, 0, kSplitHeader, s);
-  if (e != cudaSuccess) return e;
-  auto hk = k_part_hist<K>;
-  auto sk = k_part_scatter<K, V, RegionMap, kVals>;
-  const size_t hsm = static_cast<size_t>(kHistWarps) * m.R * sizeof(unsigned int);
-  const size_t ssm = scatter_smem_bytes<K, V>();
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(hk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kHistWarps * kMaxRegions * 4));
-    cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ssm));
-    attr = true;
-  }
-  const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
-  const unsigned hg = static_cast<unsigned>(std::min<uint64_t>(
-      (n + kPartTile - 1) / kPartTile, static_cast<uint64_t>(occupancy_smem(hk, kPartThreads, hsm)) * t->sm_count));
-  const unsigned sg = static_cast<unsigned>(
-      std::min<uint64_t>(ntiles, static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count));
-  hk<<<hg, kPartThreads, hsm, s>>>(keys, n, m, hist);
-  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, pk, pv,
-                                   reinterpret_cast<uint2*>(sc + extra_off + runs_at));
-  e = cudaGetLastError();
-  out.keys = pk;
-  out.vals = pv;
+  out.hist = hist;
   out.counters = reinterpret_cast<unsigned long long*>(sc + kSplitCnt);
   out.extra = sc + extra_off;
-  return e;
+  e = cudaMemsetAsync(sc, 0, kSplitHeader, s);
+  if (e != cudaSuccess) return e;
+  return split_launch<K, V, kVals, kItems>(t, m, keys, vals, n, hist,
+                                           reinterpret_cast<unsigned int*>(sc + kSplitCursor), const_cast<K*>(out.keys),
+                                           const_cast<V*>(out.vals), reinterpret_cast<uint2*>(out.extra + runs_at), s);
 }
 
 }  // namespace wc

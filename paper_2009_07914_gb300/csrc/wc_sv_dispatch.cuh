@@ -51,8 +51,9 @@ cudaError_t sv_insert_op(const wc_table* t, const void* keys, const void* vals, 
     return launch_k(t, kern, g.blocks, block, 0, s, d, k, static_cast<const Val*>(vals), n, g.per_warp,
                     static_cast<unsigned long long*>(nullptr), 0u);
   RegionSplit<Key, Val> sp;
-  cudaError_t e = vals != nullptr ? region_split(t, lc.region_mib, k, static_cast<const Val*>(vals), n, s, sp)
-                                  : region_split<Key, Val, kValsOne>(t, lc.region_mib, k, nullptr, n, s, sp);
+  const RegionMap m = region_map(t, lc.region_mib);
+  cudaError_t e = vals != nullptr ? region_split(t, m, k, static_cast<const Val*>(vals), n, s, sp)
+                                  : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp);
   if (e != cudaSuccess) return e;
   const unsigned grid = static_cast<unsigned>(bps) * static_cast<unsigned>(t->sm_count);
   e = launch_k(t, kern, grid, block, 0, s, d, sp.keys, sp.vals, n, static_cast<uint64_t>(0), sp.counters, 512u);
