@@ -198,8 +198,9 @@ typedef struct {
  * a group loads the windows of two keys, so twice as many random window reads are in
  * flight per warp (single-value retrieves of up to 32 bytes of window per lane; elsewhere
  * it is taken as 1).  Default 2 for lookups of 4+4-byte single-value tables, else 1.
- * Lookups of windows of at most 64 bytes run one query per thread, whatever group_size,
- * block_threads, blocks_per_sm and keys_in_flight say (WC_SCHEME_DEDUP keeps the group). */
+ * Inserts into and lookups of windows of at most 64 bytes run one key per thread, whatever
+ * group_size, block_threads, blocks_per_sm and keys_in_flight say (WC_SCHEME_DEDUP keeps the
+ * group); erases, wider windows and multi-value tables take them as they are. */
 typedef struct {
   int32_t group_size;
   int32_t block_threads;

@@ -57,7 +57,8 @@ typedef struct {
   int32_t reserved;
   int32_t group_insert;   /* lanes per key of inserts (0 = 2 for W 8 and 16, 1 for W 4);
                              W 4: 1 or 2, W 8: 1, 2 or 4, W 16: 2 or 4 -- e.g. the autotuner's
-                             direct-insert choice for the tables' key width and load */
+                             direct-insert choice for the tables' key width and load.  Windows
+                             of 4 and 8 slots are filled and looked up one key per thread */
   int32_t group_retrieve; /* lanes per key of lookups and erases (0 = 2, 4 for W 16); same sets */
 } wc_executor_config;
 

@@ -12,7 +12,9 @@
 #include "wc.h"
 #include "wc_exec.h"
 #include "wc_internal.h"
+#include "wc_insert.cuh"
 #include "wc_launch.cuh"
+#include "wc_lookup.cuh"
 #include "wc_sv_kernels.cuh"
 
 namespace wc {
@@ -79,8 +81,9 @@ __device__ bool wait_group(const unsigned long long* gtiles, const unsigned long
   }
 }
 
-// Lanes per key per operation (packed 64-bit slots): GI for inserts, GR for lookups and
-// erases; the kernel is instantiated for every valid pair of each window width.
+// Windows of at most 64 bytes are looked up and filled one key per thread (wc_lookup.cuh,
+// wc_insert.cuh); wider ones with GI lanes per key for inserts and GR for lookups, erases
+// with GR lanes per key.  The kernel is instantiated for every valid pair of each width.
 template <int W, int GI, int GR>
 __global__ void __launch_bounds__(kExecThreads, 3) k_exec(const ExecHeader* __restrict__ hdr,
                                                        const unsigned long long* __restrict__ gtiles,
@@ -92,7 +95,13 @@ __global__ void __launch_bounds__(kExecThreads, 3) k_exec(const ExecHeader* __re
                                                        uint64_t timeout_ns) {
   using L = LayoutP32;
   constexpr int SI = W / GI, SR = W / GR;
+  constexpr bool kOne = lookup_window<L>(W);  // one key per thread
+  union Queue {
+    LookupQueue<uint32_t> look;
+    InsertQueue<uint32_t, uint32_t> put;
+  };
   __shared__ uint64_t s_tb[kMaxExecItems];
+  __shared__ Queue s_q[kOne ? kExecThreads / 32 : 1];
   const uint32_t nitems = hdr->nitems;
   const uint64_t total = hdr->total_tiles;
   for (uint32_t i = threadIdx.x; i < nitems; i += kExecThreads) s_tb[i] = items[i].tile_begin;
@@ -121,20 +130,34 @@ __global__ void __launch_bounds__(kExecThreads, 3) k_exec(const ExecHeader* __re
     if (ok) {
       const uint64_t begin = (tile - it.tile_begin) * it.tile_keys;
       const uint64_t end = begin + it.tile_keys < it.n ? begin + it.tile_keys : it.n;
-      RangeSrc src(begin, end);
       uint32_t flags = 0;
       long long delta = 0;
-      if (op == WC_OP_INSERT) {
-        sv_insert_range<L, GI, SI>(t, static_cast<const uint32_t*>(it.keys), static_cast<const uint32_t*>(it.vals),
-                                   src, flags, delta);
-      } else if (op == WC_OP_RETRIEVE) {
-        EmitValue<L> emit{static_cast<uint32_t*>(it.out), it.found, nullptr};
-        sv_retrieve_range<L, GR, SR>(t, static_cast<const uint32_t*>(it.keys), src, emit, flags);
-      } else {
+      const auto* keys = static_cast<const uint32_t*>(it.keys);
+      const auto* vals = static_cast<const uint32_t*>(it.vals);
+      auto* out = static_cast<uint32_t*>(it.out);
+      if (op == WC_OP_ERASE) {
+        RangeSrc src(begin, end);
         NoOnErase none;
         long long removed = 0;
-        sv_erase_range<L, GR, SR>(t, static_cast<const uint32_t*>(it.keys), src, flags, removed, none);
+        sv_erase_range<L, GR, SR>(t, keys, src, flags, removed, none);
         delta = -removed;
+      } else if constexpr (kOne) {  // positions inside the tile, buffers from its start
+        BatchBlocks blocks(static_cast<uint32_t>(end - begin));
+        Queue& q = s_q[threadIdx.x >> 5];
+        if (op == WC_OP_INSERT) {
+          insert_blocks<L, W>(t, keys + begin, vals + begin, blocks, q.put, flags, delta);
+        } else {
+          const EmitLookup<L> emit{out + begin, it.found ? it.found + begin : nullptr, nullptr};
+          lookup_blocks<L, W>(t, keys + begin, blocks, q.look, emit, flags);
+        }
+      } else {
+        RangeSrc src(begin, end);
+        if (op == WC_OP_INSERT) {
+          sv_insert_range<L, GI, SI>(t, keys, vals, src, flags, delta);
+        } else {
+          EmitValue<L> emit{out, it.found, nullptr};
+          sv_retrieve_range<L, GR, SR>(t, keys, src, emit, flags);
+        }
       }
       flush_flags(t.status, flags);
       flush_delta(t.size, delta);
@@ -203,15 +226,19 @@ void free_executor(wc_executor* ex) {
   delete ex;
 }
 
-// The kernel of (W, GI, GR), or nullptr for a pair outside the instantiated sets.
+// The kernel of (W, GI, GR), or nullptr for a pair outside the valid sets.  Inserts of
+// windows of at most 64 bytes (W 4 and 8) do not depend on GI.
 void* kernel_for(int W, int GI, int GR) {
+  const bool valid = W == 4 ? GI == 1 || GI == 2 : W == 8 && (GI == 1 || GI == 2 || GI == 4);
+#define WC_EXEC_ONE(Wv, R) \
+  if (W == (Wv) && valid && GR == (R)) return reinterpret_cast<void*>(k_exec<Wv, 1, R>);
 #define WC_EXEC_K(Wv, I, R) \
   if (W == (Wv) && GI == (I) && GR == (R)) return reinterpret_cast<void*>(k_exec<Wv, I, R>);
-  WC_EXEC_K(4, 1, 1) WC_EXEC_K(4, 1, 2) WC_EXEC_K(4, 2, 1) WC_EXEC_K(4, 2, 2)
-  WC_EXEC_K(8, 1, 1) WC_EXEC_K(8, 1, 2) WC_EXEC_K(8, 1, 4) WC_EXEC_K(8, 2, 1) WC_EXEC_K(8, 2, 2)
-  WC_EXEC_K(8, 2, 4) WC_EXEC_K(8, 4, 1) WC_EXEC_K(8, 4, 2) WC_EXEC_K(8, 4, 4)
+  WC_EXEC_ONE(4, 1) WC_EXEC_ONE(4, 2)
+  WC_EXEC_ONE(8, 1) WC_EXEC_ONE(8, 2) WC_EXEC_ONE(8, 4)
   WC_EXEC_K(16, 2, 2) WC_EXEC_K(16, 2, 4) WC_EXEC_K(16, 4, 2) WC_EXEC_K(16, 4, 4)
 #undef WC_EXEC_K
+#undef WC_EXEC_ONE
   return nullptr;
 }
 

@@ -1,0 +1,265 @@
+// Inserts into windows of at most 64 bytes: one pair per thread, straight-line, like the
+// lookups of wc_lookup.cuh.
+//
+// Swept region by region (or into a table that fits L2) an insert is bound by the L2's rate
+// of window reads followed by CASes (ldcg1 ff. in wc_device.cuh: 68 G/s at best) and by its
+// chain of those two round trips.  The first window of a key takes most of them, so it is
+// probed straight from the input; pairs that are not placed there (a full window, a lost
+// race for a slot) go to the warp's queue in shared memory and are worked on 32 at a time.
+// The claim rules are those of sv_insert_range (the group-per-key engine that wider windows
+// run on): the earliest candidate of the key's sequence once the walk has met an empty slot
+// or its end.
+//
+// The sweep of 2^27 pairs, one GB300, that engine against this kernel (with half-line
+// reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.86 ms, at 0.5 3.11 -> 2.30;
+// 8+8 bytes at 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.  In input order, 2^20
+// pairs at 0.9 65.7 -> 65.6 us, at 0.5 44.0 -> 40.1; half a table erased and inserted again
+// (2^20 keys, 0.9) 172 -> 118 us.
+#pragma once
+
+#include "wc_launch.cuh"
+#include "wc_lookup.cuh"
+#include "wc_sv_kernels.cuh"
+
+namespace wc {
+
+// What an insert needs to know of a window.
+struct Spot {
+  uint32_t at;    // slot of the key (hit)
+  uint32_t tomb;  // first tombstone (has_tomb)
+  uint32_t used;  // slots that are not empty: the empty ones are the last ones (probe_window)
+  bool hit, has_tomb;
+};
+
+// S slots, the first of them slot `first` of the window, in one word: bit 0 the key is here,
+// bit 1 a tombstone is, bits 2..7 the key's slot, 8..13 the first tombstone, 14.. slots in use.
+template <class L, int S>
+__device__ __forceinline__ uint32_t spot_word(const typename L::Slot (&s)[S], typename L::Key k, uint32_t first) {
+  uint32_t hit = 0, tomb = 0, used = 0;
+#pragma unroll
+  for (int i = S - 1; i >= 0; --i) {
+    const typename L::Key kk = L::key(s[i]);
+    if (kk == k) hit = 1u | (first + i) << 2;
+    if (kk == L::kTomb) tomb = 2u | (first + i) << 8;
+    if (kk != L::kEmpty) used += 1u << 14;
+  }
+  return hit | tomb | used;
+}
+
+// Window w seen by the key k in every lane with `on`; every lane of the warp calls.  As in
+// probe_window, a pair of lanes reads a 64-byte window in one request.
+template <class L, int W>
+__device__ __forceinline__ Spot spot_of(const typename L::Slot* slots, bool on, typename L::Key k, uint32_t w) {
+  using Slot = typename L::Slot;
+  w = on ? w : 0u;  // a lane without a key reads the first window
+  uint32_t lo, hi = 0;  // the window's first half (or all of it), its second
+  if constexpr (W * slot_size<L>() <= 32) {
+    Slot s[W];
+    load_slots<L, W, true>(slots + static_cast<uint64_t>(w) * W, s);
+    lo = spot_word<L, W>(s, k, 0);
+  } else {
+    constexpr int S = W / 2;
+    const bool odd = threadIdx.x & 1;
+    const uint32_t ow = __shfl_xor_sync(kFull, w, 1);
+    const typename L::Key ok = __shfl_xor_sync(kFull, k, 1);
+    const uint32_t half = odd ? S : 0;
+    Slot sa[S], sb[S];  // my half of the even lane's window and of the odd lane's
+    load_slots<L, S, true>(slots + static_cast<uint64_t>(odd ? ow : w) * W + half, sa);
+    load_slots<L, S, true>(slots + static_cast<uint64_t>(odd ? w : ow) * W + half, sb);
+    const uint32_t ma = spot_word<L, S>(sa, odd ? ok : k, half), mb = spot_word<L, S>(sb, odd ? k : ok, half);
+    const uint32_t o = __shfl_xor_sync(kFull, odd ? ma : mb, 1);  // mine, as the other lane sees it
+    lo = odd ? o : ma;
+    hi = odd ? mb : o;
+  }
+  Spot r;
+  r.hit = (lo | hi) & 1u;
+  r.has_tomb = (lo | hi) & 2u;
+  r.at = ((lo | hi) >> 2) & 63u;  // the key is in one half at most
+  r.tomb = ((lo & 2u ? lo : hi) >> 8) & 63u;
+  r.used = (lo >> 14) + (hi >> 14);
+  return r;
+}
+
+// One slot, bypassing L1.
+template <class L>
+__device__ __forceinline__ typename L::Slot slot_now(const typename L::Slot* p) {
+  if constexpr (L::kHalf) {
+    return typename L::Slot{__ldcg(reinterpret_cast<const uint32_t*>(p))};
+  } else {
+    typename L::Slot s[1];
+    load_slots<L, 1, true>(p, s);
+    return s[0];
+  }
+}
+
+template <class Key, class Val>
+struct InsertQueue {
+  Key key[kWarpQueue];
+  Val val[kWarpQueue];
+  uint32_t w[kWarpQueue], j[kWarpQueue];
+  uint64_t tomb[kWarpQueue];
+};
+
+// The inserts of a warp's blocks; every lane calls.  vals == nullptr: every value is 1 (sets;
+// counting tables without weights).  added: new keys stored by this lane.
+template <class L, int W>
+__device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename L::Key* __restrict__ keys,
+                                              const typename L::Val* __restrict__ vals, BatchBlocks& blocks,
+                                              InsertQueue<typename L::Key, typename L::Val>& q, uint32_t& flags,
+                                              long long& added) {
+  using Slot = typename L::Slot;
+  using Key = typename L::Key;
+  using Val = typename L::Val;
+  // first tombstone of a walk: none; none, and the pair has lost a slot before; its index,
+  // with kReread when the pair has lost a slot before
+  constexpr uint64_t kNone = ~0ull, kLost = ~1ull, kReread = 1ull << 62;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  Slot* slots = static_cast<Slot*>(t.slots);
+  uint32_t cnt = 0;
+
+  // A pair on its walk: hash h, window w, the j-th of the sequence, `tomb` the first
+  // tombstone met before it.
+  struct Pair {
+    Key k;
+    Val v;
+    uint32_t w, j;
+    uint64_t tomb, h;
+  };
+  // One window of the walk, in every lane with `on` (cleared when the pair is done).  A free
+  // slot is taken to hold the word that clears and erases leave; a pair that has lost a slot
+  // reads the word again before its CAS.
+  auto step = [&](bool& on, Pair& x) {
+    const Spot s = spot_of<L, W>(slots, on, x.k, x.w);
+    if (!on) return;
+    const uint64_t base = static_cast<uint64_t>(x.w) * W;
+    if (s.hit) {  // overwrite the value (duplicate warning, Sec. IV-B3)
+      slot_store_value<L>(slots, t.vals, base + s.at, x.v);
+      if constexpr (!L::kCount) flags |= kFlagDuplicate;
+      on = false;
+      return;
+    }
+    // A pair that lost a slot has walked to its end without meeting the key, so the first
+    // free slot it meets now is its own: had a copy of the key gone to a later window since,
+    // it would have passed that free slot (tombstones only get fewer during an insert).
+    const bool at_once = x.tomb == kLost && s.has_tomb;
+    if (s.has_tomb && x.tomb >= kLost) x.tomb = (base + s.tomb) | (x.tomb == kLost ? kReread : 0ull);
+    const bool from_tomb = x.tomb < kLost;
+    if (s.used == W && x.j + 1 < t.p && !at_once) {  // no empty slot: walk on
+      if (t.ovf != nullptr) ovf_mark(t.ovf, x.w, static_cast<uint32_t>(x.h) & 7u);
+      x.w = probe_next(x.w, 1u + __umulhi(static_cast<uint32_t>(x.h), t.p - 1u), t.p);
+      ++x.j;
+      return;
+    }
+    if (!from_tomb && s.used == W) {
+      flags |= kFlagProbeLimit;  // every window visited, nothing to claim
+      on = false;
+      return;
+    }
+    // claim the earliest candidate: the remembered tombstone, else the first empty slot
+    const uint64_t c = from_tomb ? x.tomb & ~kReread : base + s.used;
+    Slot old = from_tomb ? L::tomb() : Slot{};
+    bool ok = true;
+    if (from_tomb ? (x.tomb & kReread) != 0 : x.tomb == kLost) {
+      old = slot_now<L>(slots + c);
+      ok = L::key(old) == (from_tomb ? L::kTomb : L::kEmpty);
+    }
+    if (ok) ok = L::cas(slots + c, old, L::make(x.k, x.v));
+    if (ok) {
+      if constexpr (L::kSoA) slot_store_value<L>(slots, t.vals, c, x.v);
+      ++added;
+      on = false;
+      return;
+    }
+    // another pair took it: on from the slot's window (the ones before it hold no free slot)
+    x.w = static_cast<uint32_t>(c / W);
+    if (from_tomb) x.j = 0;
+    x.tomb = kLost;
+  };
+  auto enqueue = [&](bool yes, const Pair& x) {
+    const uint32_t b = __ballot_sync(kFull, yes);
+    if (yes) {
+      const uint32_t at = cnt + __popc(b & below);
+      q.key[at] = x.k;
+      q.val[at] = x.v;
+      q.w[at] = x.w;
+      q.j[at] = x.j;
+      q.tomb[at] = x.tomb;
+    }
+    cnt += __popc(b);
+    __syncwarp();
+  };
+  // a step for the last (at most 32) pairs of the queue
+  auto drain = [&]() {
+    const uint32_t m = cnt < 32 ? cnt : 32;
+    cnt -= m;
+    bool on = lane < m;
+    Pair x{};
+    if (on) {
+      x.k = q.key[cnt + lane];
+      x.v = q.val[cnt + lane];
+      x.w = q.w[cnt + lane];
+      x.j = q.j[cnt + lane];
+      x.tomb = q.tomb[cnt + lane];
+    }
+    __syncwarp();
+    x.h = fmix64(static_cast<uint64_t>(x.k) ^ t.seed);
+    step(on, x);
+    enqueue(on, x);
+  };
+
+  const uint32_t nn = blocks.n;
+  uint32_t base = blocks.take();
+  Key kn = nn - base > lane ? ldg_stream(keys + base + lane) : Key(0);
+  Val vn = vals == nullptr ? Val(1) : nn - base > lane ? ldg_stream(vals + base + lane) : Val(0);
+  while (base != nn) {
+    const Key k = kn;
+    const Val v = vn;
+    const bool in = nn - base > lane, bad = in && is_sentinel(k);
+    base = blocks.take();
+    kn = nn - base > lane ? ldg_stream(keys + base + lane) : Key(0);  // the next block's pairs
+    if (vals != nullptr) vn = nn - base > lane ? ldg_stream(vals + base + lane) : Val(0);
+    // counting inserts run on aggregated batches whose padding is key 0 (the aggregation
+    // pass already flagged the caller's sentinel keys)
+    if (bad && !(L::kCount && k == Key(0))) flags |= kFlagInvalid;
+    Pair x{k, v, 0, 0, kNone, fmix64(static_cast<uint64_t>(k) ^ t.seed)};  // as probe_init
+    x.w = __umulhi(static_cast<uint32_t>(x.h >> 32), t.p);
+    bool on = in && !bad;
+    step(on, x);
+    enqueue(on, x);
+    while (cnt >= 32) drain();
+  }
+  while (cnt > 0) drain();
+}
+
+// counter != nullptr: a batch split by table region, swept in order.
+template <class L, int W>
+__global__ void __launch_bounds__(kLookThreads, 4)
+    k_insert(TableDesc t, const typename L::Key* __restrict__ keys, const typename L::Val* __restrict__ vals,
+             uint64_t n, unsigned long long* counter) {
+  __shared__ InsertQueue<typename L::Key, typename L::Val> q[kLookThreads / 32];
+  uint32_t flags = 0;
+  long long added = 0;
+  BatchBlocks blocks(n, counter);
+  insert_blocks<L, W>(t, keys, vals, blocks, q[threadIdx.x >> 5], flags, added);
+  flush_flags(t.status, flags);
+  flush_delta(t.size, added);
+}
+
+// Batches below 2^21 pairs into a table that is not swept run three blocks per SM: with more,
+// the pairs in flight are about as many as a table of their size has windows, and what is
+// lost in races for slots is more than the latency hidden (2^20 pairs at load 0.9, 3 / 4 / 5
+// blocks: 65.6 / 70.6 / 77.0 us; at load 0.5 40.1 / 43.4 / 45.8; 2^22 at 0.9 129 / 121 / 124).
+template <class L, int W>
+cudaError_t insert_launch(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
+                          unsigned long long* counter, cudaStream_t s) {
+  auto kern = k_insert<L, W>;
+  int per_sm = occupancy(kern, kLookThreads);
+  if (counter == nullptr && n < (1ull << 21)) per_sm = std::min(per_sm, 3);
+  const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
+  const uint64_t most = static_cast<uint64_t>(per_sm) * t->sm_count;
+  return launch_k(t, kern, static_cast<unsigned>(std::min(want, most)), kLookThreads, 0, s, desc_of(t), keys, vals, n,
+                  counter);
+}
+
+}  // namespace wc

@@ -134,44 +134,57 @@ __device__ __forceinline__ Probe<L> probe_window(const typename L::Slot* slots, 
   return r;
 }
 
-// counter != nullptr: warps take chunks of kLookChunk queries in order from it (a batch
-// sorted by table region); otherwise blocks of 32 queries are strided over the grid.
-template <class L, int W, class Emit, class KIn = typename L::Key>
-__global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const KIn* __restrict__ keys, uint64_t n,
-                                                            unsigned long long* counter, Emit emit) {
-  using Slot = typename L::Slot;
-  using Key = typename L::Key;
-  constexpr int kQueue = 64;  // at most 31 left over + 32 of one step
-  __shared__ KIn q_key[kLookThreads / 32][kQueue];
-  __shared__ uint32_t q_pos[kLookThreads / 32][kQueue], q_w[kLookThreads / 32][kQueue], q_j[kLookThreads / 32][kQueue];
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t below = (1u << lane) - 1u;
-  const Slot* slots = static_cast<const Slot*>(t.slots);
-  uint32_t flags = 0, cnt = 0;
-
-  // warp-uniform: the next block of 32 queries (n < 2^32), and the end of the taken chunk
-  const uint32_t nn = static_cast<uint32_t>(n), stride = gridDim.x * kLookThreads;
-  uint32_t next = counter != nullptr ? nn : (blockIdx.x * kLookThreads + threadIdx.x) & ~31u;
-  uint32_t chunk_end = counter != nullptr ? nn : 0xffffffffu;
-  // first query of the next block, n when there is none
-  auto take = [&]() -> uint32_t {
+// A warp's blocks of 32 consecutive inputs (warp-uniform).  counter != nullptr: chunks of
+// kLookChunk inputs are taken from it in order, so the grid sweeps the batch front to back;
+// otherwise the blocks are strided over the grid.  Inputs are numbered in 32 bits (n < 2^32).
+struct BatchBlocks {
+  uint32_t n, next, end;  // end of the taken chunk
+  uint32_t stride;
+  unsigned long long* counter;
+  __device__ __forceinline__ BatchBlocks(uint64_t n_, unsigned long long* c)
+      : n(static_cast<uint32_t>(n_)), next(c != nullptr ? n : (blockIdx.x * blockDim.x + threadIdx.x) & ~31u), end(n),
+        stride(gridDim.x * blockDim.x), counter(c) {}
+  // all of n inputs for this warp (one tile of the batched executor)
+  __device__ __forceinline__ explicit BatchBlocks(uint32_t n_) : n(n_), next(0), end(n_), stride(32), counter(nullptr) {}
+  // first input of the next block, n when there is none
+  __device__ __forceinline__ uint32_t take() {
     if (counter == nullptr) {
       const uint32_t b = next;
-      next = nn - b > stride && b < nn ? b + stride : nn;
-      return b < nn ? b : nn;
+      next = b < n && n - b > stride ? b + stride : n;
+      return b < n ? b : n;
     }
-    if (next >= chunk_end) {
+    if (next >= end) {
       unsigned long long c = 0;
-      if (lane == 0) c = atomicAdd(counter, static_cast<unsigned long long>(kLookChunk));
+      if ((threadIdx.x & 31) == 0) c = atomicAdd(counter, static_cast<unsigned long long>(kLookChunk));
       c = __shfl_sync(kFull, c, 0);
-      if (c >= n) return nn;  // and again: the counter only grows
+      if (c >= n) return n;  // and so every time from now on: the counter only grows
       next = static_cast<uint32_t>(c);
-      chunk_end = n - c > kLookChunk ? next + kLookChunk : nn;
+      end = n - next > kLookChunk ? next + kLookChunk : n;
     }
     const uint32_t b = next;
-    next = chunk_end - b > 32 ? b + 32 : chunk_end;
+    next = end - b > 32 ? b + 32 : end;
     return b;
-  };
+  }
+};
+
+// A warp's queue of open queries: at most 31 left over + 32 of one step.
+constexpr int kWarpQueue = 64;
+template <class KIn>
+struct LookupQueue {
+  KIn key[kWarpQueue];
+  uint32_t pos[kWarpQueue], w[kWarpQueue], j[kWarpQueue];
+};
+
+// The lookups of a warp's blocks; every lane calls.
+template <class L, int W, class Emit, class KIn>
+__device__ __forceinline__ void lookup_blocks(const TableDesc& t, const KIn* __restrict__ keys, BatchBlocks& blocks,
+                                              LookupQueue<KIn>& q, const Emit& emit, uint32_t& flags) {
+  using Slot = typename L::Slot;
+  using Key = typename L::Key;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  const Slot* slots = static_cast<const Slot*>(t.slots);
+  uint32_t cnt = 0;
 
   // one step for the last (at most 32) queries of the queue: the next window of their
   // sequence, and where that is full its overflow bit
@@ -183,10 +196,10 @@ __global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const K
     KIn kin = 0;
     uint32_t pos = 0, w = 0, j = 0;
     if (on) {
-      kin = q_key[wid][cnt + lane];
-      pos = q_pos[wid][cnt + lane];
-      w = q_w[wid][cnt + lane];
-      j = q_j[wid][cnt + lane] + 1;
+      kin = q.key[cnt + lane];
+      pos = q.pos[cnt + lane];
+      w = q.w[cnt + lane];
+      j = q.j[cnt + lane] + 1;
     }
     __syncwarp();
     const Key k = static_cast<Key>(kin);
@@ -201,22 +214,23 @@ __global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const K
     const uint32_t b = __ballot_sync(kFull, again);
     if (again) {
       const uint32_t at = cnt + __popc(b & below);
-      q_key[wid][at] = kin;
-      q_pos[wid][at] = pos;
-      q_w[wid][at] = w;
-      q_j[wid][at] = j;
+      q.key[at] = kin;
+      q.pos[at] = pos;
+      q.w[at] = w;
+      q.j[at] = j;
     }
     cnt += __popc(b);
     if (on && !again) emit(pos, r.hit, r.v, static_cast<uint64_t>(w) * W + r.sub);
   };
 
-  uint32_t base = take();
+  const uint32_t nn = blocks.n;
+  uint32_t base = blocks.take();
   KIn kn = nn - base > lane ? ldg_stream(keys + base + lane) : KIn(0);
   while (base != nn) {
     const KIn kin = kn;
     const bool in = nn - base > lane;
     const uint32_t pos = base + lane;
-    base = take();
+    base = blocks.take();
     kn = nn - base > lane ? ldg_stream(keys + base + lane) : KIn(0);  // the next block's queries
     const bool bad = in && is_sentinel(kin);
     if (bad) flags |= kFlagInvalid;
@@ -231,16 +245,26 @@ __global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const K
     const uint32_t b = __ballot_sync(kFull, open);
     if (open) {
       const uint32_t at = cnt + __popc(b & below);
-      q_key[wid][at] = kin;
-      q_pos[wid][at] = pos;
-      q_w[wid][at] = w;
-      q_j[wid][at] = 0;
+      q.key[at] = kin;
+      q.pos[at] = pos;
+      q.w[at] = w;
+      q.j[at] = 0;
     }
     cnt += __popc(b);
     if (in && !open) emit(pos, r.hit, r.v, static_cast<uint64_t>(w) * W + r.sub);
     while (cnt >= 32) drain();
   }
   while (cnt > 0) drain();
+}
+
+// counter != nullptr: a batch sorted by table region, swept in order.
+template <class L, int W, class Emit, class KIn = typename L::Key>
+__global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const KIn* __restrict__ keys, uint64_t n,
+                                                            unsigned long long* counter, Emit emit) {
+  __shared__ LookupQueue<KIn> q[kLookThreads / 32];
+  uint32_t flags = 0;
+  BatchBlocks blocks(n, counter);
+  lookup_blocks<L, W>(t, keys, blocks, q[threadIdx.x >> 5], emit, flags);
   flush_flags(t.status, flags);
 }
 

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_oa_insert(TableDesc t, const typename L
     uint32_t mm = 0, me = 0, mt = 0;
     const uint64_t lane_slot = static_cast<uint64_t>(w) * W + ln.r * S;
     if (act) {
-      load_slots<L, S>(slots + lane_slot, s);
+      load_slots<L, S, true>(slots + lane_slot, s);
       classify<L, S>(s, k, mm, me, mt);
     }
     const uint32_t fr = me | mt;
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) k_oa_erase(TableDesc t, const typename L:
     uint32_t mm = 0, me = 0, mt = 0;
     const uint64_t lane_slot = static_cast<uint64_t>(w) * W + ln.r * S;
     if (act) {
-      load_slots<L, S>(slots + lane_slot, s);
+      load_slots<L, S, true>(slots + lane_slot, s);
       classify<L, S>(s, k, mm, me, mt);
 #pragma unroll
       for (int i = 0; i < S; ++i)

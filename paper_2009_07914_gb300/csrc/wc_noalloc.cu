@@ -24,7 +24,7 @@
 #include "wc_internal.h"
 #include "wc_launch.cuh"
 #include "wc_partition.cuh"
-#include "wc_sv_kernels.cuh"
+#include "wc_sv_dispatch.cuh"
 
 namespace wc {
 namespace {
@@ -103,14 +103,10 @@ cudaError_t run(const wc_table* t, const void* keys, const void* vals, uint64_t 
   Val* pv = reinterpret_cast<Val*>(sc + kHeadBytes + (n * sizeof(Key) + 255) / 256 * 256);
   cudaError_t e = cudaMemsetAsync(sc, 0, kWorkOff + 8, s);
   if (e != cudaSuccess) return e;
-  auto ik = k_sv_insert<L, G, S, H>;
   e = split_launch<Key, Val>(t, m, static_cast<const Key*>(keys), static_cast<const Val*>(vals), n, hist, cursor, pk,
                              pv, nullptr, s);
   if (e != cudaSuccess) return e;  // no insert over a split that was never written
-  const int block = lc.block_threads;
-  const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : occupancy(ik, block);
-  return launch_k(t, ik, static_cast<unsigned>(bps) * static_cast<unsigned>(t->sm_count), block, 0, s, desc_of(t),
-                  static_cast<const Key*>(pk), static_cast<const Val*>(pv), n, static_cast<uint64_t>(0), work, 512u);
+  return insert_kernel<L, G, S, H>(t, pk, pv, n, work, s);
 }
 
 #define WC_NA_CASE(L, Wv, Gv) \

@@ -1,6 +1,7 @@
 // Instantiation and dispatch of the single-value kernels for one slot layout.
 #pragma once
 
+#include "wc_insert.cuh"
 #include "wc_launch.cuh"
 #include "wc_lookup.cuh"
 #include "wc_partition.cuh"
@@ -34,29 +35,40 @@ cudaError_t sv_retrieve_blocked(const wc_table* t, const wc_launch& lc, const ty
   return e != cudaSuccess ? e : r;
 }
 
+// The insert kernel of a window: counter != nullptr for a batch split by region.
+template <class L, int G, int S, int H = 1>
+cudaError_t insert_kernel(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
+                          unsigned long long* counter, cudaStream_t s) {
+  if constexpr (lookup_window<L>(G * S * H)) {
+    return insert_launch<L, G * S * H>(t, keys, vals, n, counter, s);
+  } else {
+    const wc_launch& lc = t->launch[WC_OP_INSERT];
+    auto kern = k_sv_insert<L, G, S, H>;
+    const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : occupancy(kern, lc.block_threads);
+    const EngineGrid g = engine_grid(n, G, lc.block_threads, bps, t->sm_count);
+    const unsigned grid =
+        counter != nullptr ? static_cast<unsigned>(bps) * static_cast<unsigned>(t->sm_count) : g.blocks;
+    return launch_k(t, kern, grid, lc.block_threads, 0, s, desc_of(t), keys, vals, n, g.per_warp, counter,
+                    counter != nullptr ? kLookChunk : 0u);
+  }
+}
+
 // Insert (direct, or the blocked scheme: split the batch by table region, then insert it
 // region by region).  vals == nullptr (counting tables): every key counts 1.
 template <class L, int G, int S, int H = 1>
 cudaError_t sv_insert_op(const wc_table* t, const void* keys, const void* vals, uint64_t n, cudaStream_t s) {
   using Key = typename L::Key;
   using Val = typename L::Val;
+  constexpr int W = G * S * H;
   const wc_launch& lc = t->launch[WC_OP_INSERT];
-  const int block = lc.block_threads;
-  const TableDesc d = desc_of(t);
   const Key* k = static_cast<const Key*>(keys);
-  auto kern = k_sv_insert<L, G, S, H>;
-  const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : occupancy(kern, block);
-  const EngineGrid g = engine_grid(n, G, block, bps, t->sm_count);
-  if (scheme_for(t, WC_OP_INSERT, n) != WC_SCHEME_BLOCKED)
-    return launch_k(t, kern, g.blocks, block, 0, s, d, k, static_cast<const Val*>(vals), n, g.per_warp,
-                    static_cast<unsigned long long*>(nullptr), 0u);
+  const Val* v = static_cast<const Val*>(vals);
+  if (scheme_for(t, WC_OP_INSERT, n) != WC_SCHEME_BLOCKED) return insert_kernel<L, G, S, H>(t, k, v, n, nullptr, s);
   RegionSplit<Key, Val> sp;
   const RegionMap m = region_map(t, lc.region_mib);
-  cudaError_t e = vals != nullptr ? region_split(t, m, k, static_cast<const Val*>(vals), n, s, sp)
-                                  : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp);
-  if (e != cudaSuccess) return e;
-  const unsigned grid = static_cast<unsigned>(bps) * static_cast<unsigned>(t->sm_count);
-  e = launch_k(t, kern, grid, block, 0, s, d, sp.keys, sp.vals, n, static_cast<uint64_t>(0), sp.counters, 512u);
+  cudaError_t e = v != nullptr ? region_split(t, m, k, v, n, s, sp)
+                               : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp);
+  if (e == cudaSuccess) e = insert_kernel<L, G, S, H>(t, sp.keys, sp.vals, n, sp.counters, s);
   const cudaError_t r = scratch_release(t, s);
   return e != cudaSuccess ? e : r;
 }

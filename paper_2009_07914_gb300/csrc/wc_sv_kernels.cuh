@@ -556,7 +556,7 @@ __device__ __forceinline__ void sv_insert_range(const TableDesc& t, const typena
     uint32_t mm = 0, me = 0, mt = 0;
     const uint64_t lane_slot = static_cast<uint64_t>(w) * W + Steps<H>::offset(h, SW) + ln.r * S;
     if (act) {
-      load_slots<L, S>(slots + lane_slot, s);
+      load_slots<L, S, true>(slots + lane_slot, s);
       classify<L, S>(s, k, mm, me, mt);
     }
     const uint32_t bm = group_vote<G>(mm != 0, ln.gbase);
@@ -703,7 +703,7 @@ __device__ __forceinline__ void sv_erase_range(const TableDesc& t, const KIn* __
     uint32_t mm = 0, me = 0, mt = 0;
     const uint64_t lane_slot = static_cast<uint64_t>(w) * W + Steps<H>::offset(h, SW) + ln.r * S;
     if (act) {
-      load_slots<L, S>(slots + lane_slot, s);
+      load_slots<L, S, true>(slots + lane_slot, s);
       classify<L, S>(s, k, mm, me, mt);
     }
     const uint32_t bm = group_vote<G>(mm != 0, ln.gbase);

@@ -1,0 +1,100 @@
+"""Inserts one pair per thread, in input order and swept by region: the sizes where a warp's
+block, its queue and a chunk of the sweep begin and end, repeated keys, tombstones that many
+pairs want at once, and a table that is filled to its last slot -- against the oracle's plain
+map and the reachability check of the slot dump."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import wc_inputs
+
+pytestmark = pytest.mark.gpu
+
+SEED = 0x5EED_C0DE
+
+
+@pytest.fixture(scope="module")
+def wc():
+    from paper_2009_07914_gb300 import build
+    build.build()
+    import paper_2009_07914_gb300 as m
+    return m
+
+
+def _inputs(kb, n, seed):
+    if kb == 4:
+        return wc_inputs.distinct_u32(seed, n), wc_inputs.uniform_u32(seed + 1, n)
+    return wc_inputs.distinct_u64(seed, n), wc_inputs.uniform_u64(seed + 1, n)
+
+
+def _same(wc, t, o, q):
+    out, found, _ = t.retrieve(q)
+    eo, ef, _ = o.retrieve(q)
+    np.testing.assert_array_equal(found, ef)
+    np.testing.assert_array_equal(out, eo)
+    assert t.size() == o.size()
+
+
+def _layout(wc, t, soa):
+    from paper_2009_07914_gb300 import api
+    if soa:
+        return
+    i = t.info
+    bits = api.wc_table_dump_overflow_bits(t.handle) if i["options"] & wc.WC_OPT_OVERFLOW_BITS else None
+    r = oracle.check_slots(api.wc_table_dump_slots(t.handle), i["windows"], i["window_width"], i["slot_bytes"], SEED,
+                           True, bits)
+    assert r["dups"] == 0 and r["unreachable"] == 0
+
+
+@pytest.mark.parametrize("blocked", [False, True], ids=["direct", "swept"])
+@pytest.mark.parametrize("kb,W,soa,bits", [(4, 8, 0, 1), (4, 4, 0, 0), (8, 4, 0, 1), (8, 2, 0, 0), (4, 16, 1, 0),
+                                           (8, 8, 1, 0)])
+def test_batches_erases_and_reinserts(wc, kb, W, soa, bits, blocked):
+    opt = (wc.WC_OPT_SOA if soa else 0) | (wc.WC_OPT_OVERFLOW_BITS if bits else 0)
+    for n in (1, 31, 33, 511, 513, 4097, 60_013):
+        keys, vals = _inputs(kb, n + 64, 0x1A5 + n)
+        t = wc.SingleValueTable(kb, kb, min_capacity=int(n / 0.95) + 1, window_width=W, options=opt, seed=SEED)
+        if blocked:
+            lc = wc.wc_table_get_launch(t.handle, wc.WC_OP_INSERT)
+            t.set_launch(wc.WC_OP_INSERT, lc["group_size"], scheme=wc.WC_SCHEME_BLOCKED, region_mib=1)
+        o = oracle.SingleValue(kb, kb)
+        k = keys[:n].copy()
+        if n > 100:
+            k[50] = 0
+            k[51] = 2 ** (8 * kb) - 1
+        assert t.insert(k, vals[:n]) == o.insert(k, vals[:n])
+        _same(wc, t, o, keys)
+        t.erase(k[::2])
+        o.erase(k[::2])
+        # the erased keys with new values; what is stored already is overwritten
+        again, v2 = np.concatenate([k[::2], k[1::4]]), wc_inputs.uniform_u64(n, n)[:k[::2].size + k[1::4].size]
+        v2 = v2.astype(vals.dtype)
+        assert t.insert(again, v2) == o.insert(again, v2)
+        _same(wc, t, o, keys)
+        _layout(wc, t, soa)
+
+
+@pytest.mark.parametrize("kb,W", [(4, 8), (8, 4)])
+def test_last_slots_and_repeats(wc, kb, W):
+    """More distinct keys than slots, in a table full of tombstones: every slot is taken, the
+    rest raises PROBE_LIMIT; each key of a batch of repeats is stored once, with one of its
+    values."""
+    t = wc.SingleValueTable(kb, kb, min_capacity=5 * W, window_width=W, seed=SEED)
+    cap = t.capacity
+    keys, vals = _inputs(kb, cap + 40, 0x7A8)
+    t.insert(keys[:cap], vals[:cap])
+    t.erase(keys[:cap])
+    assert t.size() == 0
+    flags = t.insert(keys, vals)
+    assert flags & wc.WC_FLAG_PROBE_LIMIT and t.size() == cap
+    out, found, _ = t.retrieve(keys)
+    assert found.sum() == cap and np.array_equal(out[found == 1], vals[found == 1])
+    big = wc.SingleValueTable(kb, kb, min_capacity=1 << 12, window_width=W, seed=SEED)
+    pick = np.arange(200_000) % 997
+    v = np.arange(200_000).astype(vals.dtype)
+    k = _inputs(kb, 997, 0x99)[0][pick]
+    assert big.insert(k, v) == wc.WC_FLAG_DUPLICATE_KEY and big.size() == 997
+    out, found, _ = big.retrieve(k[:997])
+    assert found.all() and np.array_equal(out.astype(np.int64) % 997, pick[:997])
