@@ -178,8 +178,16 @@ def ptr(x) -> int | None:
     raise TypeError("expected a torch.Tensor or an integer device address, got %r" % type(x))
 
 
+# The current stream's handle without the Stream object that torch.cuda.current_stream()
+# builds for it: 0.2 us against 2.9 us, of a call whose native part takes 4 us.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def stream_handle(stream) -> int | None:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream

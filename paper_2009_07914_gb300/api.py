@@ -27,17 +27,19 @@ __all__ = [
 
 
 def _n_of(n, t: torch.Tensor | None, width: int | None = None) -> int:
-    if n is None:
-        if not isinstance(t, torch.Tensor):
-            raise ValueError("n is required when the keys are a raw address")
-        n = t.numel()
     if isinstance(t, torch.Tensor):
-        if t.numel() < n:
-            raise ValueError("buffer holds %d elements, n = %d" % (t.numel(), n))
-        if width is not None and t.numel() and t.element_size() != width:
-            raise ValueError("element width %d, table expects %d" % (t.element_size(), width))
-        if t.numel() and not t.is_cuda:
-            raise ValueError("device buffers must be CUDA tensors")
+        m = t.numel()
+        if n is None:
+            n = m
+        elif m < n:
+            raise ValueError("buffer holds %d elements, n = %d" % (m, n))
+        if m:
+            if width is not None and t.element_size() != width:
+                raise ValueError("element width %d, table expects %d" % (t.element_size(), width))
+            if not t.is_cuda:
+                raise ValueError("device buffers must be CUDA tensors")
+    elif n is None:
+        raise ValueError("n is required when the keys are a raw address")
     return int(n)
 
 
