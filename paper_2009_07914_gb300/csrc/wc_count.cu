@@ -28,10 +28,13 @@ bool count_shape_ok(int slot_bytes, int W, int G) {
 namespace {
 
 // Pass before the insert: each block sums the weights of equal keys inside a tile of
-// kCntTile inputs in a shared-memory table and writes the tile's distinct keys with their
-// sums to the front of the tile's range of the output, key 0 (skipped by the counting
-// insert) behind them -- a hot key then costs one atomic add per tile instead of one per
-// occurrence.  Sentinel inputs raise INVALID_KEY here.
+// kCntTile inputs in a shared-memory table -- a hot key then costs one atomic add per tile
+// instead of one per occurrence.  With a cursor (zeroed by the caller) the distinct keys of
+// all tiles are written one behind the other, their number left in it: the passes that
+// follow then only see those (2^26 Zipf draws over 2^24 keys: 34 M of 67 M; the padding went
+// to one region of the split).  Without one they go to the front of the tile's range of the
+// output, key 0 (skipped by the counting insert) behind them.  Sentinel inputs raise
+// INVALID_KEY here.
 constexpr int kCntThreads = 512;
 constexpr int kCntItems = 8;
 constexpr int kCntTile = kCntThreads * kCntItems;
@@ -45,11 +48,12 @@ constexpr size_t count_agg_smem() {
 template <class K, class V>
 __global__ void __launch_bounds__(kCntThreads) k_count_aggregate(const K* __restrict__ keys, const V* __restrict__ w,
                                                                  uint64_t n, K* __restrict__ ok, V* __restrict__ ov,
-                                                                 uint32_t* status) {
+                                                                 uint32_t* status, unsigned long long* cursor) {
   extern __shared__ unsigned long long cnt_smem[];
   K* s_key = reinterpret_cast<K*>(cnt_smem);
   V* s_sum = reinterpret_cast<V*>(s_key + kCntSlots);
   __shared__ uint32_t s_warp[kCntThreads / 32];
+  __shared__ unsigned long long s_base;
   uint32_t flags = 0;
   const uint64_t ntiles = (n + kCntTile - 1) / kCntTile;
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -100,29 +104,42 @@ __global__ void __launch_bounds__(kCntThreads) k_count_aggregate(const K* __rest
       if (q < warp) pos += s_warp[q];
       total += s_warp[q];
     }
+    uint64_t base = t0;
+    if (cursor != nullptr) {
+      if (threadIdx.x == 0) s_base = atomicAdd(cursor, static_cast<unsigned long long>(total));
+      __syncthreads();
+      base = s_base;
+    }
 #pragma unroll
     for (int q = 0; q < per; ++q) {
       const int e = q * kCntThreads + threadIdx.x;
       if (s_key[e] != K(0)) {
-        ok[t0 + pos] = s_key[e];
-        ov[t0 + pos] = s_sum[e];
+        ok[base + pos] = s_key[e];
+        ov[base + pos] = s_sum[e];
         ++pos;
       }
     }
-    for (uint32_t i = total + threadIdx.x; i < tn; i += kCntThreads) ok[t0 + i] = K(0);  // padding
+    if (cursor == nullptr)
+      for (uint32_t i = total + threadIdx.x; i < tn; i += kCntThreads) ok[t0 + i] = K(0);  // padding
     __syncthreads();
   }
   if (flags) atomicOr(status, flags);
 }
 
+// The aggregated batch in the table's scratch, behind skip_bytes: [its size 256 B | keys |
+// sums].  dense: one key behind the other, *n_dev = where their number is (else null).
 template <class K, class V>
 cudaError_t aggregate(const wc_table* t, const void* keys, const void* weights, uint64_t n, uint64_t skip_bytes,
-                      const void** akeys, const void** avals, cudaStream_t s) {
+                      bool dense, const void** akeys, const void** avals, const unsigned long long** n_dev,
+                      cudaStream_t s) {
   const uint64_t kbytes = (n * sizeof(K) + 255) / 256 * 256;
-  cudaError_t e = ensure_scratch(t, skip_bytes + kbytes + n * sizeof(V), s);
+  cudaError_t e = ensure_scratch(t, skip_bytes + 256 + kbytes + n * sizeof(V), s);
   if (e != cudaSuccess) return e;
-  K* ok = reinterpret_cast<K*>(static_cast<char*>(t->d_scratch) + skip_bytes);
+  auto* cursor = reinterpret_cast<unsigned long long*>(static_cast<char*>(t->d_scratch) + skip_bytes);
+  K* ok = reinterpret_cast<K*>(reinterpret_cast<char*>(cursor) + 256);
   V* ov = reinterpret_cast<V*>(reinterpret_cast<char*>(ok) + kbytes);
+  if (dense) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
   auto kern = k_count_aggregate<K, V>;
   static bool attr = false;
   if (!attr) {
@@ -132,20 +149,21 @@ cudaError_t aggregate(const wc_table* t, const void* keys, const void* weights, 
   const uint64_t ntiles = (n + kCntTile - 1) / kCntTile;
   const uint64_t most = static_cast<uint64_t>(occupancy_smem(kern, kCntThreads, count_agg_smem<K, V>())) * t->sm_count;
   kern<<<static_cast<unsigned>(ntiles < most ? ntiles : most), kCntThreads, count_agg_smem<K, V>(), s>>>(
-      static_cast<const K*>(keys), static_cast<const V*>(weights), n, ok, ov, t->d_status);
+      static_cast<const K*>(keys), static_cast<const V*>(weights), n, ok, ov, t->d_status, dense ? cursor : nullptr);
   *akeys = ok;
   *avals = ov;
+  *n_dev = dense ? cursor : nullptr;
   return cudaGetLastError();
 }
 
 }  // namespace
 
 #define WC_COUNT_CASE(L, Wv, Gv) \
-  if (W == (Wv) && G == (Gv)) return sv_insert_op<L, (Gv), (Wv) / (Gv)>(t, keys, weights, n, s);
+  if (W == (Wv) && G == (Gv)) return sv_insert_op<L, (Gv), (Wv) / (Gv)>(t, keys, weights, n, s, n_dev);
 
-// Insert of the aggregated batch (keys, per-tile sums; key 0 = padding).
+// Insert of the aggregated batch (keys, per-tile sums; key 0 = padding where n_dev is null).
 static cudaError_t count_insert_agg(const wc_table* t, const void* keys, const void* weights, uint64_t n,
-                                    cudaStream_t s) {
+                                    const unsigned long long* n_dev, cudaStream_t s) {
   const int W = static_cast<int>(t->W);
   const int G = t->launch[WC_OP_INSERT].group_size;
   if (t->slot_bytes == 8) {
@@ -168,12 +186,17 @@ cudaError_t count_insert(const wc_table* t, const void* keys, const void* weight
   const uint64_t kb = static_cast<uint64_t>(t->cfg.key_bytes);
   const bool split = scheme_for(t, WC_OP_INSERT, n) == WC_SCHEME_BLOCKED;
   const uint64_t skip = split ? kSplitHeader + 2 * ((n * kb + 255) / 256 * 256) : 0;
+  // windows of at most 64 bytes: their insert takes a batch size from the device (a small
+  // batch is not worth the launch that zeroes it)
+  const bool dense = n >= (1ull << 18) && t->W * t->slot_bytes <= 64;
   const void* ak = nullptr;
   const void* av = nullptr;
-  cudaError_t e = kb == 4 ? aggregate<uint32_t, uint32_t>(t, keys, weights, n, skip, &ak, &av, s)
-                          : aggregate<unsigned long long, unsigned long long>(t, keys, weights, n, skip, &ak, &av, s);
+  const unsigned long long* n_dev = nullptr;
+  cudaError_t e = kb == 4 ? aggregate<uint32_t, uint32_t>(t, keys, weights, n, skip, dense, &ak, &av, &n_dev, s)
+                          : aggregate<unsigned long long, unsigned long long>(t, keys, weights, n, skip, dense, &ak,
+                                                                              &av, &n_dev, s);
   if (e != cudaSuccess) return e;
-  e = count_insert_agg(t, ak, av, n, s);
+  e = count_insert_agg(t, ak, av, n, n_dev, s);
   const cudaError_t r = scratch_release(t, s);
   return e != cudaSuccess ? e : r;
 }

@@ -225,6 +225,7 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
     Pair x{k, v, 0, 0, kNone, fmix64(static_cast<uint64_t>(k) ^ t.seed)};  // as probe_init
     x.w = __umulhi(static_cast<uint32_t>(x.h >> 32), t.p);
     bool on = in && !bad;
+    if (!__any_sync(kFull, on)) continue;  // padding of an aggregated batch
     step(on, x);
     enqueue(on, x);
     while (cnt >= 32) drain();
@@ -232,11 +233,13 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
   while (cnt > 0) drain();
 }
 
-// counter != nullptr: a batch split by table region, swept in order.
+// counter != nullptr: a batch split by table region, swept in order.  n_dev (or null): the
+// batch's size on the device, at most n.
 template <class L, int W>
 __global__ void __launch_bounds__(kLookThreads, 4)
     k_insert(TableDesc t, const typename L::Key* __restrict__ keys, const typename L::Val* __restrict__ vals,
-             uint64_t n, unsigned long long* counter) {
+             uint64_t n, unsigned long long* counter, const unsigned long long* n_dev) {
+  if (n_dev != nullptr) n = *n_dev;
   __shared__ InsertQueue<typename L::Key, typename L::Val> q[kLookThreads / 32];
   uint32_t flags = 0;
   long long added = 0;
@@ -246,20 +249,25 @@ __global__ void __launch_bounds__(kLookThreads, 4)
   flush_delta(t.size, added);
 }
 
-// Batches below 2^21 pairs into a table that is not swept run three blocks per SM: with more,
-// the pairs in flight are about as many as a table of their size has windows, and what is
-// lost in races for slots is more than the latency hidden (2^20 pairs at load 0.9, 3 / 4 / 5
-// blocks: 65.6 / 70.6 / 77.0 us; at load 0.5 40.1 / 43.4 / 45.8; 2^22 at 0.9 129 / 121 / 124).
+// Batches of 2^16 to 2^21 pairs in input order run three blocks per SM, two in tables below
+// 100,000 windows: with more, the pairs in flight outnumber the windows, and what is lost in
+// races for slots is more than the latency hidden (4+4 bytes; 2 / 3 / 5 blocks: 2^18 pairs at
+// load 0.9 47.8 / 59 / 68.7 us, at 0.5 30 / 36 / 38; 2^20 at 0.9 71.7 / 62.4 / 77.0, at 0.5
+// 44.4 / 36.5 / 45.8; 2^22 at 0.9 129 with three, 121 with four).
+inline int insert_blocks_per_sm(const wc_table* t, int most, uint64_t n, bool swept) {
+  if (swept || n <= (1ull << 16) || n >= (1ull << 21)) return most;
+  return std::min(most, t->windows < 100000 ? 2 : 3);
+}
+
 template <class L, int W>
 cudaError_t insert_launch(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
-                          unsigned long long* counter, cudaStream_t s) {
+                          unsigned long long* counter, const unsigned long long* n_dev, cudaStream_t s) {
   auto kern = k_insert<L, W>;
-  int per_sm = occupancy(kern, kLookThreads);
-  if (counter == nullptr && n < (1ull << 21)) per_sm = std::min(per_sm, 3);
+  const int per_sm = insert_blocks_per_sm(t, occupancy(kern, kLookThreads), n, counter != nullptr);
   const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
   const uint64_t most = static_cast<uint64_t>(per_sm) * t->sm_count;
   return launch_k(t, kern, static_cast<unsigned>(std::min(want, most)), kLookThreads, 0, s, desc_of(t), keys, vals, n,
-                  counter);
+                  counter, n_dev);
 }
 
 }  // namespace wc

@@ -62,8 +62,10 @@ inline uint32_t hist_copies(uint32_t R) { return R <= 512 ? kHistWarps : R <= 10
 
 template <class K>
 __global__ void __launch_bounds__(kPartThreads) k_part_hist(const K* __restrict__ keys, uint64_t n, RegionMap m,
-                                                            unsigned int* __restrict__ hist, uint32_t copies) {
+                                                            unsigned int* __restrict__ hist, uint32_t copies,
+                                                            const unsigned long long* n_dev) {
   extern __shared__ unsigned int s_hw[];  // copies * R
+  if (n_dev != nullptr) n = *n_dev;
   for (uint32_t i = threadIdx.x; i < copies * m.R; i += kPartThreads) s_hw[i] = 0;
   __syncthreads();
   unsigned int* mine = s_hw + ((threadIdx.x >> 5) & (copies - 1)) * m.R;
@@ -191,7 +193,8 @@ template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
 __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlocks))
     k_part_scatter(const K* __restrict__ keys, const V* __restrict__ vals, uint64_t n, RegionMap m,
                    const unsigned int* __restrict__ hist, unsigned int* __restrict__ cursor, K* __restrict__ okeys,
-                   V* __restrict__ ovals, uint2* __restrict__ runs) {
+                   V* __restrict__ ovals, uint2* __restrict__ runs, const unsigned long long* n_dev) {
+  if (n_dev != nullptr) n = *n_dev;
   using Tile = SplitTile<K, V, kVals>;
   constexpr bool kPre = Tile::kPre, kRead = kVals == kValsRead;
   constexpr int kTile = kPartThreads * kItems;
@@ -331,10 +334,12 @@ struct RegionSplit {
 
 inline uint64_t align256(uint64_t x) { return (x + 255) / 256 * 256; }
 
-// The two kernels of a split: hist and cursor are m.R zeroed words each.
+// The two kernels of a split: hist and cursor are m.R zeroed words each.  n_dev (or null): the
+// batch's size on the device, at most n.
 template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
 cudaError_t split_launch(const wc_table* t, const RegionMap& m, const K* keys, const V* vals, uint64_t n,
-                         unsigned int* hist, unsigned int* cursor, K* okeys, V* ovals, uint2* runs, cudaStream_t s) {
+                         unsigned int* hist, unsigned int* cursor, K* okeys, V* ovals, uint2* runs, cudaStream_t s,
+                         const unsigned long long* n_dev = nullptr) {
   auto hk = k_part_hist<K>;
   auto sk = k_part_scatter<K, V, kVals, kItems>;
   using Tile = SplitTile<K, V, kVals>;
@@ -353,10 +358,10 @@ cudaError_t split_launch(const wc_table* t, const RegionMap& m, const K* keys, c
   const uint64_t split_most = static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count;
   const unsigned hg = static_cast<unsigned>(std::min<uint64_t>((n + kPartTile - 1) / kPartTile, hist_most));
   const unsigned sg = static_cast<unsigned>(std::min<uint64_t>((n + kTile - 1) / kTile, split_most));
-  hk<<<hg, kPartThreads, hsm, s>>>(keys, n, m, hist, copies);
+  hk<<<hg, kPartThreads, hsm, s>>>(keys, n, m, hist, copies, n_dev);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;  // no split without its counts
-  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, okeys, ovals, runs);
+  sk<<<sg, kPartThreads, ssm, s>>>(keys, vals, n, m, hist, cursor, okeys, ovals, runs, n_dev);
   return cudaGetLastError();
 }
 
@@ -365,7 +370,8 @@ cudaError_t split_launch(const wc_table* t, const RegionMap& m, const K* keys, c
 // run starts to extra + runs_at).  The caller hands the scratch on with scratch_release.
 template <class K, class V, int kVals = kValsRead, int kItems = kPartItems>
 cudaError_t region_split(const wc_table* t, const RegionMap& m, const K* keys, const V* vals, uint64_t n,
-                         cudaStream_t s, RegionSplit<K, V>& out, uint64_t extra = 0, uint64_t runs_at = 0) {
+                         cudaStream_t s, RegionSplit<K, V>& out, uint64_t extra = 0, uint64_t runs_at = 0,
+                         const unsigned long long* n_dev = nullptr) {
   const uint64_t keys_off = kSplitHeader;
   const uint64_t vals_off = keys_off + align256(n * sizeof(K));
   const uint64_t extra_off = vals_off + (kVals == kValsNone ? 0 : align256(n * sizeof(V)));
@@ -382,7 +388,8 @@ cudaError_t region_split(const wc_table* t, const RegionMap& m, const K* keys, c
   if (e != cudaSuccess) return e;
   return split_launch<K, V, kVals, kItems>(t, m, keys, vals, n, hist,
                                            reinterpret_cast<unsigned int*>(sc + kSplitCursor), const_cast<K*>(out.keys),
-                                           const_cast<V*>(out.vals), reinterpret_cast<uint2*>(out.extra + runs_at), s);
+                                           const_cast<V*>(out.vals), reinterpret_cast<uint2*>(out.extra + runs_at), s,
+                                           n_dev);
 }
 
 }  // namespace wc

@@ -35,12 +35,13 @@ cudaError_t sv_retrieve_blocked(const wc_table* t, const wc_launch& lc, const ty
   return e != cudaSuccess ? e : r;
 }
 
-// The insert kernel of a window: counter != nullptr for a batch split by region.
+// The insert kernel of a window: counter != nullptr for a batch split by region.  n_dev (one
+// key per thread only, or null): the batch's size on the device, at most n.
 template <class L, int G, int S, int H = 1>
 cudaError_t insert_kernel(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
-                          unsigned long long* counter, cudaStream_t s) {
+                          unsigned long long* counter, cudaStream_t s, const unsigned long long* n_dev = nullptr) {
   if constexpr (lookup_window<L>(G * S * H)) {
-    return insert_launch<L, G * S * H>(t, keys, vals, n, counter, s);
+    return insert_launch<L, G * S * H>(t, keys, vals, n, counter, n_dev, s);
   } else {
     const wc_launch& lc = t->launch[WC_OP_INSERT];
     auto kern = k_sv_insert<L, G, S, H>;
@@ -56,19 +57,20 @@ cudaError_t insert_kernel(const wc_table* t, const typename L::Key* keys, const 
 // Insert (direct, or the blocked scheme: split the batch by table region, then insert it
 // region by region).  vals == nullptr (counting tables): every key counts 1.
 template <class L, int G, int S, int H = 1>
-cudaError_t sv_insert_op(const wc_table* t, const void* keys, const void* vals, uint64_t n, cudaStream_t s) {
+cudaError_t sv_insert_op(const wc_table* t, const void* keys, const void* vals, uint64_t n, cudaStream_t s,
+                         const unsigned long long* n_dev = nullptr) {
   using Key = typename L::Key;
   using Val = typename L::Val;
   constexpr int W = G * S * H;
   const wc_launch& lc = t->launch[WC_OP_INSERT];
   const Key* k = static_cast<const Key*>(keys);
   const Val* v = static_cast<const Val*>(vals);
-  if (scheme_for(t, WC_OP_INSERT, n) != WC_SCHEME_BLOCKED) return insert_kernel<L, G, S, H>(t, k, v, n, nullptr, s);
+  if (scheme_for(t, WC_OP_INSERT, n) != WC_SCHEME_BLOCKED) return insert_kernel<L, G, S, H>(t, k, v, n, nullptr, s, n_dev);
   RegionSplit<Key, Val> sp;
   const RegionMap m = region_map(t, lc.region_mib);
-  cudaError_t e = v != nullptr ? region_split(t, m, k, v, n, s, sp)
+  cudaError_t e = v != nullptr ? region_split(t, m, k, v, n, s, sp, 0, 0, n_dev)
                                : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp);
-  if (e == cudaSuccess) e = insert_kernel<L, G, S, H>(t, sp.keys, sp.vals, n, sp.counters, s);
+  if (e == cudaSuccess) e = insert_kernel<L, G, S, H>(t, sp.keys, sp.vals, n, sp.counters, s, n_dev);
   const cudaError_t r = scratch_release(t, s);
   return e != cudaSuccess ? e : r;
 }
