@@ -297,7 +297,7 @@ cudaError_t scratch_release(const wc_table* t, cudaStream_t s) {
 // whose hot lines stay in L2 (256 MiB, Zipf: 78 against 49); above, it wins both (1.1 GiB,
 // Zipf: 32.5 against 48.1).  8+8-byte pairs: 2.2 GiB 23.8 against 27.1, Zipf 28.8 against
 // 35.8.  Not inside a stream capture: the scratch must not belong to the graph.
-static bool lookup_splits(const wc_table* t, uint64_t n) {
+bool lookup_splits(const wc_table* t, uint64_t n) {
   return t->table_bytes > (512ull << 20) && n >= t->table_bytes / 64;
 }
 
@@ -498,13 +498,14 @@ wc_status wc_table_create(wc_table** out, const wc_table_config* cfg) {
   DeviceGuard guard(t->device);
   t->sm_count = sm_count_of(t->device);
 
-  // One allocation: [slots | meta 256 B | overflow bits (SV) | pending (MV) | scan partials (MV, OA) | pool (MV)]
+  // One allocation: [slots | meta 256 B | overflow bits (SV), walk bits (OA) | pending (MV) | scan partials (MV, OA) | pool (MV)]
   const bool sv = (cfg->kind == WC_SINGLE_VALUE || cfg->kind == WC_COUNTING || cfg->kind == WC_HASH_SET) &&
                   (cfg->options & WC_OPT_OVERFLOW_BITS);
   const uint64_t off_meta = align_up(t->table_bytes, kAlign);
   const uint64_t off_ovf = off_meta + kAlign;
   const uint64_t ovf_bytes = sv ? align_up((p + 3) / 4 * 4, kAlign) : 0;  // one byte per window
-  const uint64_t off_pending = off_ovf + ovf_bytes;
+  t->walk_bytes = oa ? align_up((p + 3) / 4 * 4, kAlign) : 0;  // one byte per window, too
+  const uint64_t off_pending = off_ovf + ovf_bytes + t->walk_bytes;
   const uint64_t pending_bytes = mv ? align_up(cap * 4, kAlign) : 0;
   const uint64_t off_base = off_pending + pending_bytes;
   const uint64_t base_bytes = growth != kGrowExact ? align_up(cap * 4, kAlign) : 0;
@@ -532,6 +533,7 @@ wc_status wc_table_create(wc_table** out, const wc_table_config* cfg) {
   t->d_nkeys = reinterpret_cast<unsigned long long*>(base + off_meta + 16);
   t->d_cursor = reinterpret_cast<unsigned long long*>(base + off_meta + 24);
   t->d_ovf = sv ? reinterpret_cast<uint32_t*>(base + off_ovf) : nullptr;
+  t->d_walk = oa ? reinterpret_cast<uint32_t*>(base + off_ovf) : nullptr;
   t->d_vals = soa ? static_cast<void*>(base + soa_vals_off) : nullptr;
   t->d_pending = mv ? reinterpret_cast<uint32_t*>(base + off_pending) : nullptr;
   t->d_base = growth != kGrowExact ? reinterpret_cast<uint32_t*>(base + off_base) : nullptr;
@@ -577,14 +579,14 @@ wc_status wc_table_create(wc_table** out, const wc_table_config* cfg) {
     cudaGetLastError();
   }
 
-  t->clear_bytes = off_partials;
+  t->clear_bytes = off_partials - t->walk_bytes;  // OA tables end their cleared prefix with the walk bits
   cudaError_t ge = cudaSuccess;
   if (t->d_growth != nullptr) {
     ge = cudaMemcpy(t->d_growth, cum_size.data(), cum_size.size() * 8, cudaMemcpyHostToDevice);
     if (ge == cudaSuccess)
       ge = cudaMemcpy(t->d_growth + t->nbuckets, cum_foot.data(), cum_foot.size() * 8, cudaMemcpyHostToDevice);
   }
-  if (ge != cudaSuccess || cudaMemset(t->d_block, 0, t->clear_bytes) != cudaSuccess ||
+  if (ge != cudaSuccess || cudaMemset(t->d_block, 0, t->clear_bytes + t->walk_bytes) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
     cudaFree(t->d_block);
     delete t;
@@ -613,7 +615,7 @@ wc_status wc_table_clear(wc_table* t, void* stream) {
   TraceRange trace("wc_table_clear");
   if (t == nullptr) return WC_ERR_INVALID_ARG;
   DeviceGuard guard(t->device);
-  return cuda_status(cudaMemsetAsync(t->d_block, 0, t->clear_bytes, as_stream(stream)));
+  return cuda_status(cudaMemsetAsync(t->d_block, 0, t->clear_bytes + t->walk_bytes, as_stream(stream)));
 }
 
 wc_status wc_table_get_info(const wc_table* t, wc_table_info* h_out) {

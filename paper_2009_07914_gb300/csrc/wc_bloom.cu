@@ -264,7 +264,7 @@ cudaError_t contains(const wc_table* t, const K* keys, uint64_t n, uint8_t* foun
     cudaError_t e = query_split(t, 0, keys, n, s, q);
     if (e == cudaSuccess) {
       e = launch_k(t, kern, static_cast<unsigned>(most), 256u, 0, s, desc_of(t), q.sp.keys, n, k, q.rf, q.sp.counters);
-      if (e == cudaSuccess) e = unsplit_launch<K, uint8_t>(t, q, n, nullptr, found, s);
+      if (e == cudaSuccess) e = unsplit_launch(t, q, n, static_cast<uint8_t*>(nullptr), found, s);
       const cudaError_t r = scratch_release(t, s);
       return e != cudaSuccess ? e : r;
     }

@@ -33,7 +33,7 @@ SnapHeader header_of(const wc_table* t) {
   h.windows = t->windows;
   h.pool_capacity = t->pool_capacity;
   h.seed = t->cfg.seed;
-  h.device_bytes = t->device_bytes;
+  h.device_bytes = t->device_bytes - t->walk_bytes;  // walk bits are not part of a snapshot
   h.clear_bytes = t->clear_bytes;
   h.bucket_first_size = t->cfg.bucket_first_size;
   std::memcpy(&h.bucket_growth_bits, &t->cfg.bucket_growth, sizeof(double));
@@ -111,6 +111,8 @@ wc_status wc_table_restore(wc_table* t, const void* h_in, uint64_t bytes, void* 
   if (e == cudaSuccess && t->d_pool)
     e = cudaMemcpyAsync(t->d_pool, src + t->clear_bytes, t->device_bytes - pool_offset(t), cudaMemcpyHostToDevice,
                         s);
+  // any pair of the snapshot may have walked past any window
+  if (e == cudaSuccess && t->d_walk != nullptr) e = cudaMemsetAsync(t->d_walk, 0xff, t->walk_bytes, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return wc::cuda_status(e);
 }
@@ -125,6 +127,7 @@ wc_status wc_table_device_view(const wc_table* t, wc_device_view* h_out) {
   // per-element appends need buckets of known sizes (a growth strategy) and pool offsets
   // below bit 63 of the list handle, which marks a list whose next bucket is being made
   if (bl && (t->growth == wc::kGrowExact || t->pool_capacity >= (1ull << 34))) return WC_ERR_UNSUPPORTED;
+  t->walk_off = true;
   *h_out = wc_device_view{};
   h_out->slots = t->d_slots;
   h_out->status = t->d_status;

@@ -118,6 +118,7 @@ struct wc_table {
   uint64_t pool_capacity;
   uint64_t device_bytes;
   uint64_t clear_bytes;  // prefix of d_block zeroed by a clear (slots, meta, pending)
+  uint64_t walk_bytes;   // OA: walk bits, also zeroed, behind that prefix
   void* d_block;         // the single allocation holding everything below
   void* d_slots;
   uint32_t* d_status;
@@ -125,6 +126,8 @@ struct wc_table {
   unsigned long long* d_nkeys;
   unsigned long long* d_cursor;
   uint32_t* d_ovf;       // SV: overflow bits, one byte per window
+  uint32_t* d_walk;      // OA: walk bits, one byte per window
+  mutable bool walk_off = false;  // the slots were handed to user kernels: the walk bits may miss pairs
   void* d_vals;          // SoA single-value tables: value array (capacity entries)
   uint32_t* d_pending;   // MV: capacity entries
   uint32_t* d_base;      // MV with bucket growth: capacity entries
@@ -201,6 +204,9 @@ int scheme_for(const wc_table* t, int op, uint64_t n);
 
 // The same for lookups, on stream s.
 int lookup_scheme(const wc_table* t, uint64_t n, cudaStream_t s);
+
+// Whether a batch of n lookups is worth splitting by table region.
+bool lookup_splits(const wc_table* t, uint64_t n);
 
 // Scratch a split lookup of n queries takes (0: it would not be split): an insert of as
 // many pairs grows the buffer to it, so the lookup after it does not have to grow it again.

@@ -278,10 +278,10 @@ __global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const K
 // split batch and in the tile's own region order), so the block of a tile reads the tile's
 // R runs, puts every result at its input position (lidx) in shared memory and writes the
 // tile out in order -- no scattered store leaves the SM.
-template <class V>
+template <class V, class Out = V>
 __global__ void __launch_bounds__(kPartThreads, 3) k_unsplit(const uint16_t* __restrict__ lidx, const V* __restrict__ rv,
                                                           const uint8_t* __restrict__ rf, uint64_t n, uint32_t R,
-                                                          const uint2* __restrict__ runs, V* __restrict__ out,
+                                                          const uint2* __restrict__ runs, Out* __restrict__ out,
                                                           uint8_t* __restrict__ found) {
   __shared__ V s_v[kPartTile];
   __shared__ __align__(4) uint8_t s_f[kPartTile];
@@ -393,10 +393,10 @@ cudaError_t query_split(const wc_table* t, int region_mib, const K* keys, uint64
   return cudaSuccess;
 }
 
-template <class K, class V>
-cudaError_t unsplit_launch(const wc_table* t, const QuerySplit<K, V>& q, uint64_t n, V* out, uint8_t* found,
+template <class K, class V, class Out = V>
+cudaError_t unsplit_launch(const wc_table* t, const QuerySplit<K, V>& q, uint64_t n, Out* out, uint8_t* found,
                            cudaStream_t s) {
-  auto kern = k_unsplit<V>;
+  auto kern = k_unsplit<V, Out>;
   const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
   const unsigned grid = static_cast<unsigned>(
       std::min<uint64_t>(ntiles, static_cast<uint64_t>(occupancy(kern, kPartThreads)) * t->sm_count));
