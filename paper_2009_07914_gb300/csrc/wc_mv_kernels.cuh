@@ -164,48 +164,33 @@ struct Agg {
 // ones: the key could not be stored), their number at len[tile], and for every element
 // elem[e] = (position of its key in the list) << 16 | (its rank among the tile's elements
 // of that key), or all ones for a sentinel key.
+// block_base (exact layout, or null): pool start of what each block of pass 2 allocated; the
+// pending counters then count from the run's place behind it, so that a reservation is one
+// atomic and the handle is not read (70 M random reads of 2^28 Zipf inserts).
 struct TileRecord {
   uint2* list;
   uint32_t* elem;
   uint32_t* len;
+  uint64_t* block_base;
 };
 
+// Entry of a key in the tile's table; fresh: this lane put it there.
 template <int kSlots>
-__device__ __forceinline__ int smem_find_or_insert(unsigned long long* s_key, unsigned long long key) {
+__device__ __forceinline__ int smem_find_or_insert(unsigned long long* s_key, unsigned long long key, bool& fresh) {
   volatile unsigned long long* vk = s_key;
-  uint32_t h = static_cast<uint32_t>(fmix64(key) >> 40) & (kSlots - 1);
+  // Fibonacci hashing: the table lives for one tile, and the keys of a tile come from
+  // everywhere (a full mix cost more than the few collisions it saves)
+  uint32_t h = static_cast<uint32_t>((key * 0x9E3779B97F4A7C15ull) >> 40) & (kSlots - 1);
   while (true) {  // at most kSlots / 2 distinct keys in a table of kSlots slots
     const unsigned long long cur = vk[h];
     if (cur == key) return static_cast<int>(h);
     if (cur == 0ull) {
       const unsigned long long prev = atomicCAS(s_key + h, 0ull, key);
+      fresh = prev == 0ull;
       if (prev == 0ull || prev == key) return static_cast<int>(h);
     }
     h = (h + 1) & (kSlots - 1);
   }
-}
-
-// Exclusive block scan of one uint32 per thread; total gets the sum.
-template <int kThreads>
-__device__ __forceinline__ uint32_t block_exclusive_u32(uint32_t x, uint32_t& total, uint32_t* s_w) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t inc = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFull, inc, o);
-    if (lane >= o) inc += y;
-  }
-  if (lane == 31) s_w[warp] = inc;
-  __syncthreads();
-  uint32_t before = 0;
-  total = 0;
-#pragma unroll
-  for (int w = 0; w < kThreads / 32; ++w) {
-    if (w < warp) before += s_w[w];
-    total += s_w[w];
-  }
-  __syncthreads();
-  return before + inc - x;
 }
 
 // The global phase of one tile: every distinct key of the tile (s_list[0..len)) is found
@@ -318,7 +303,6 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
   unsigned short* s_pos = reinterpret_cast<unsigned short*>(s_ks + kAggTile);  // list position of every table entry
   unsigned short* s_list = s_pos + kAggSlots;  // the tile's distinct keys (table entries), kAggTile
   KIn* s_in = reinterpret_cast<KIn*>(reinterpret_cast<char*>(agg_smem) + Agg<kAggThreads>::table_bytes());
-  __shared__ uint32_t s_wsum[kAggThreads / 32];
   __shared__ uint32_t s_len, s_next;
   const int lane = threadIdx.x & 31;
   const uint64_t ntiles = (n + kAggTile - 1) / kAggTile;
@@ -345,10 +329,18 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
     if (tile_counter != nullptr) {
       if (threadIdx.x == 0) s_ntile = atomicAdd(tile_counter, 1ull);
     }
-    for (int e = threadIdx.x; e < kAggSlots; e += kAggThreads) {
-      s_key[e] = 0ull;
-      s_cnt[e] = 0u;
-      if (e < kAggTile) s_ks[e] = ~0u;
+    {
+      const uint4 zero = make_uint4(0, 0, 0, 0), ones = make_uint4(~0u, ~0u, ~0u, ~0u);
+      auto* k4 = reinterpret_cast<uint4*>(s_key);
+      auto* c4 = reinterpret_cast<uint4*>(s_cnt);
+      auto* l4 = reinterpret_cast<uint4*>(s_ks);
+#pragma unroll
+      for (int e = threadIdx.x; e < kAggSlots / 2; e += kAggThreads) k4[e] = zero;
+#pragma unroll
+      for (int e = threadIdx.x; e < kAggSlots / 4; e += kAggThreads) c4[e] = zero;
+#pragma unroll
+      for (int e = threadIdx.x; e < kAggTile / 4; e += kAggThreads) l4[e] = ones;
+      if (threadIdx.x == 0) s_len = s_next = 0;
     }
     cp_async_wait_all();
     __syncthreads();
@@ -374,14 +366,30 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
         if (valid) key = static_cast<unsigned long long>(kin);
         else flags |= kFlagInvalid;
       }
-      // equal keys of the warp are counted by their lowest lane
-      const uint32_t peers = __match_any_sync(kFull, key);
+      // A hot key shows up as the warp's first one: its copies are counted by their lowest
+      // lane.  The rest count one by one (grouping every key of the warp with
+      // __match_any_sync cost more than the atomics it saved).
+      const unsigned long long first = __shfl_sync(kFull, key, 0);  // every lane shuffles
+      uint32_t peers = __ballot_sync(kFull, valid && key == first);
+      if (__popc(peers) < 6 || !((peers >> lane) & 1u)) peers = 1u << lane;
       const int leader = __ffs(peers) - 1;
       int slot = -1;
       uint32_t base = 0;
+      bool fresh = false;
       if (valid && lane == leader) {
-        slot = smem_find_or_insert<kAggSlots>(s_key, key);
+        slot = smem_find_or_insert<kAggSlots>(s_key, key, fresh);
         base = atomicAdd(s_cnt + slot, static_cast<uint32_t>(__popc(peers)));
+      }
+      // the tile's distinct keys are listed as they come (their order is of no consequence)
+      const uint32_t news = __ballot_sync(kFull, fresh);
+      if (news != 0) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&s_len, static_cast<uint32_t>(__popc(news)));
+        at = __shfl_sync(kFull, at, 0) + __popc(news & ((1u << lane) - 1u));
+        if (fresh) {
+          s_list[at] = static_cast<unsigned short>(slot);
+          s_pos[slot] = static_cast<unsigned short>(at);
+        }
       }
       slot = __shfl_sync(kFull, slot, leader);
       base = __shfl_sync(kFull, base, leader);
@@ -389,33 +397,6 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
       my_rank[k] = base + __popc(peers & ((1u << lane) - 1u));
     }
     __syncthreads();
-    // compact the tile's distinct keys into a list, then probe them warp-uniformly; a
-    // thread takes every kAggThreads-th table entry, so a warp reads consecutive entries
-    // (the list order is of no consequence)
-    {
-      constexpr int kPer = kAggSlots / kAggThreads;
-      uint32_t c = 0;
-      bool used[kPer];
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        used[i] = s_key[i * kAggThreads + threadIdx.x] != 0ull;
-        c += used[i];
-      }
-      uint32_t total = 0;
-      uint32_t pos = block_exclusive_u32<kAggThreads>(c, total, s_wsum);
-#pragma unroll
-      for (int i = 0; i < kPer; ++i)
-        if (used[i]) {
-          const int e = i * kAggThreads + threadIdx.x;
-          s_pos[e] = static_cast<unsigned short>(pos);
-          s_list[pos++] = static_cast<unsigned short>(e);
-        }
-      if (threadIdx.x == 0) {
-        s_len = total;
-        s_next = 0;
-      }
-      __syncthreads();
-    }
     {
       // the record of this tile for the placing pass: element words now (the list
       // positions are known), the (slot, count) list after the key-store phase
@@ -442,6 +423,10 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
   flush_flags(t.status, flags);
   flush_delta(t.nkeys, created);
 }
+
+constexpr int kAllocThreads = 256;
+constexpr int kAllocItems = 8;
+constexpr int kAllocSlots = kAllocThreads * kAllocItems;  // key-store slots of a block of pass 2
 
 // ---- pass 3: placing the values ------------------------------------------------------------
 // With the counting pass's record of every tile (TileRecord), no key is looked up again:
@@ -496,7 +481,9 @@ __global__ void __launch_bounds__(kThreads) k_mv_place(TableDesc t, PoolDesc pd,
     for (int k = 0; k < kPer; ++k) {
       const bool ok = r[k].x != ~0u;
       old[k] = ok ? atomicAdd(pd.pending + r[k].x, r[k].y) : kPoison;
-      handle[k] = ok ? slots[r[k].x].v : 0ull;
+      handle[k] = !ok ? 0ull
+                  : rec.block_base != nullptr ? __ldg(rec.block_base + r[k].x / kAllocSlots)
+                                              : slots[r[k].x].v;
       c0[k] = ok && pd.growth != kGrowExact ? pd.base[r[k].x] : 0u;
     }
 #pragma unroll
@@ -507,7 +494,9 @@ __global__ void __launch_bounds__(kThreads) k_mv_place(TableDesc t, PoolDesc pd,
         s_b[i] = ~0ull;
         continue;
       }
-      if (pd.growth == kGrowExact) {
+      if (rec.block_base != nullptr) {
+        s_b[i] = handle[k] + old[k];
+      } else if (pd.growth == kGrowExact) {
         s_b[i] = h_offset(handle[k]) + (h_prev(handle[k]) ? Hdr<VB>::kElems : 0) + old[k];
       } else {
         // growth: `old` is the value number of the run's first value; the handle and the
@@ -537,9 +526,6 @@ __global__ void __launch_bounds__(kThreads) k_mv_place(TableDesc t, PoolDesc pd,
 }
 
 // ---- pass 2: bucket allocation ----------------------------------------------------------
-
-constexpr int kAllocThreads = 256;
-constexpr int kAllocItems = 8;
 
 // Exclusive block scan of one uint64 per thread; returns this thread's prefix and the
 // block total through `total`.
@@ -572,7 +558,8 @@ __device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t x, uint64_t& t
 }
 
 template <int VB>
-__global__ void __launch_bounds__(kAllocThreads) k_mv_alloc(TableDesc t, PoolDesc pd, uint64_t capacity) {
+__global__ void __launch_bounds__(kAllocThreads) k_mv_alloc(TableDesc t, PoolDesc pd, uint64_t capacity,
+                                                             uint64_t* block_base) {
   using V = typename PoolT<VB>::T;
   __shared__ uint64_t s_warp[kAllocThreads / 32];
   __shared__ unsigned long long s_block_base;
@@ -611,6 +598,7 @@ __global__ void __launch_bounds__(kAllocThreads) k_mv_alloc(TableDesc t, PoolDes
     const unsigned long long b = total ? atomicAdd(pd.cursor, static_cast<unsigned long long>(total)) : 0ull;
     s_block_base = b;
     s_ok = b + total <= pd.capacity;
+    if (block_base != nullptr) block_base[blockIdx.x] = b;
   }
   __syncthreads();
   long long added = 0;
@@ -627,7 +615,10 @@ __global__ void __launch_bounds__(kAllocThreads) k_mv_alloc(TableDesc t, PoolDes
     const uint64_t old = h_count(h[k]);
     if (old) *reinterpret_cast<unsigned long long*>(static_cast<V*>(pd.pool) + off) = h[k];
     slots[s].v = h_make(off, old + c[k], old != 0);
-    pd.pending[s] = 0u;  // becomes the bucket's fill cursor for pass 3
+    // becomes the bucket's fill cursor for pass 3
+    pd.pending[s] = block_base != nullptr
+                        ? static_cast<uint32_t>(off - s_block_base + (old ? Hdr<VB>::kElems : 0))
+                        : 0u;
     added += c[k];
     off += need[k];
   }
@@ -640,7 +631,8 @@ __global__ void __launch_bounds__(kAllocThreads) k_mv_alloc(TableDesc t, PoolDes
 // c0 + c - 1); they are allocated as one chunk, their headers written, the handle pointed
 // at bucket b1.  pending[s] and base[s] become c0: pass 3 counts value numbers from there.
 template <int VB>
-__global__ void __launch_bounds__(kAllocThreads) k_mv_alloc_growth(TableDesc t, PoolDesc pd, uint64_t capacity) {
+__global__ void __launch_bounds__(kAllocThreads) k_mv_alloc_growth(TableDesc t, PoolDesc pd, uint64_t capacity,
+                                                                    uint64_t*) {
   using V = typename PoolT<VB>::T;
   __shared__ uint64_t s_warp[kAllocThreads / 32];
   __shared__ unsigned long long s_block_base;
