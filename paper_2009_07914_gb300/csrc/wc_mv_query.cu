@@ -1,5 +1,6 @@
 // Multi-value queries: count_values (+ scan), retrieve_multi, erase.
 #include "wc_launch.cuh"
+#include "wc_lookup.cuh"
 #include "wc_mv_kernels.cuh"
 
 namespace wc {
@@ -15,16 +16,46 @@ bool mv_shape_ok(int W, int G) {
 
 namespace {
 
+// A row's number of values, for the lookups of wc_lookup.cuh over the key store.
+template <class Out>
+struct EmitValues {
+  Out* __restrict__ out;
+  __device__ __forceinline__ void operator()(uint32_t pos, bool hit, KsL::Val handle, uint64_t) const {
+    out[pos] = hit ? static_cast<Out>(h_count(handle)) : Out(0);
+  }
+};
+
+// Counts run one query per thread in windows of at most 64 bytes (2^24 + 2^22 queries of a
+// 320 MiB key store 0.51 -> 0.47 ms, 2^26 + 2^24 of a 1.3 GiB one 2.82 -> 1.89, 2^20 + 2^18 of
+// 20 MiB 47 -> 36 us), else on the group engine.
 template <class KIn, int G, int S>
 cudaError_t probe_op(const wc_table* t, int op, const void* keys, uint64_t n, uint64_t* offs, cudaStream_t s) {
   const TableDesc d = desc_of(t);
   const KIn* k = static_cast<const KIn*>(keys);
   const int block = t->launch[op].block_threads;
   if (op == WC_OP_COUNT) {
-    auto kern = k_mv_count<KIn, G, S>;
-    const int bps = t->launch[op].blocks_per_sm > 0 ? t->launch[op].blocks_per_sm : occupancy(kern, block);
-    const EngineGrid g = engine_grid(n, G, block, bps, t->sm_count);
-    return launch_k(t, kern, g.blocks, block, 0, s, d, k, n, g.per_warp, offs);
+    constexpr int W = G * S;
+    if constexpr (lookup_window<KsL>(W)) {
+      // split by region like lookups (lookup_splits): counts of 32 bits, widened on the way back
+      if (lookup_splits(t, n) && !stream_capturing(s)) {
+        QuerySplit<KIn, uint32_t> q;
+        cudaError_t e = query_split(t, 0, k, n, s, q);
+        if (e == cudaSuccess) {
+          e = lookup_launch<KsL, W>(t, q.sp.keys, n, q.sp.counters, EmitValues<uint32_t>{q.rv}, s);
+          if (e == cudaSuccess) e = unsplit_launch<KIn, uint32_t, uint64_t>(t, q, n, offs, nullptr, s);
+          const cudaError_t r = scratch_release(t, s);
+          return e != cudaSuccess ? e : r;
+        }
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();  // no room for the split: count in input order
+      }
+      return lookup_launch<KsL, W>(t, k, n, nullptr, EmitValues<uint64_t>{offs}, s);
+    } else {
+      auto kern = k_mv_count<KIn, G, S>;
+      const int bps = t->launch[op].blocks_per_sm > 0 ? t->launch[op].blocks_per_sm : occupancy(kern, block);
+      const EngineGrid g = engine_grid(n, G, block, bps, t->sm_count);
+      return launch_k(t, kern, g.blocks, block, 0, s, d, k, n, g.per_warp, offs);
+    }
   }
   auto kern = k_mv_erase<KIn, G, S>;
   const int bps = t->launch[op].blocks_per_sm > 0 ? t->launch[op].blocks_per_sm : occupancy(kern, block);

@@ -66,12 +66,16 @@ def test_edges_hot_keys_restore_and_view(wc, kb, W):
         assert t.size() == 0 and not t.count_values(q)[0].any()
 
 
-def test_counts_split_by_region(wc):
+@pytest.mark.parametrize("bucket", [False, True], ids=["open_addressing", "bucket"])
+def test_counts_split_by_region(wc, bucket):
     import torch
     from paper_2009_07914_gb300 import api
-    t = wc.MultiValueOATable(4, 4, min_capacity=70_000_000)
-    assert t.info["table_bytes"] > 512 << 20
     n = 3_000_017
+    if bucket:
+        t = wc.MultiValueTable(4, 4, min_capacity=36_000_000, value_pool_capacity=8 * n)
+    else:
+        t = wc.MultiValueOATable(4, 4, min_capacity=70_000_000)
+    assert t.info["table_bytes"] > 512 << 20
     keys = torch.from_numpy(wc_inputs.distinct_u32(0xC0, n).view(np.int32)).cuda()
     api.wc_insert(t.handle, keys.repeat(3), torch.arange(3 * n, device="cuda", dtype=torch.int32))
     m = t.info["table_bytes"] // 64 + 77
