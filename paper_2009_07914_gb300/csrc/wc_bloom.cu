@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(256) k_bloom_insert(TableDesc t, const K* __re
 // with 512 threads: one block of a 128 KiB region fills an SM), 1.91 ms with the split,
 // against 3.89 ms by k_bloom_insert and 6.65 ms with its former 32-bit words.
 constexpr int kFillThreads = 1024;
+constexpr uint32_t fill_words(uint32_t R) { return scan_cnt_words(R) + 2 * scan_off_words(R); }
 
 template <class K>
 __global__ void __launch_bounds__(kFillThreads) k_bloom_fill(TableDesc t, const K* __restrict__ keys, RegionMap m,
@@ -115,21 +116,17 @@ __global__ void __launch_bounds__(kFillThreads) k_bloom_fill(TableDesc t, const 
   const uint32_t words = 4u << m.shift;  // 64-bit words of a region
   unsigned long long* s_bits = fill_smem;
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(fill_smem + words);
-  uint32_t* s_off = s_cnt + m.R;   // first key of every region
-  uint32_t* s_unit = s_off + m.R;  // first unit of every region (part, region)
+  uint32_t* s_off = s_cnt + scan_cnt_words(m.R);   // first key of every region
+  uint32_t* s_unit = s_off + scan_off_words(m.R);  // first unit of every region (part, region)
   __shared__ uint32_t s_w[kFillThreads / 32];  // scan_regions: the first kPartThreads threads do the work
-  __shared__ uint32_t s_total;
   __shared__ unsigned long long s_next;
-  for (uint32_t r = threadIdx.x; r < m.R; r += kFillThreads) s_cnt[r] = hist[r];
+  for (uint32_t r = threadIdx.x; r < scan_cnt_words(m.R); r += kFillThreads) s_cnt[r] = r < m.R ? hist[r] : 0u;
   __syncthreads();
-  scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t) { s_off[r] = before; });
+  scan_regions(s_cnt, s_off, m.R, s_w);
   for (uint32_t r = threadIdx.x; r < m.R; r += kFillThreads) s_cnt[r] = (s_cnt[r] + part - 1) / part;
   __syncthreads();
-  scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t c) {
-    s_unit[r] = before;
-    if (r == m.R - 1) s_total = before + c;
-  });
-  const uint32_t units = s_total;
+  scan_regions(s_cnt, s_unit, m.R, s_w);
+  const uint32_t units = s_unit[m.R];
   uint32_t flags = 0;
   long long added = 0;
   while (true) {
@@ -230,9 +227,9 @@ cudaError_t insert(const wc_table* t, const K* keys, uint64_t n, cudaStream_t s)
     if (e == cudaSuccess) {
       if (fill) {
         auto kern = k_bloom_fill<K>;
-        const size_t smem = (32ull << m.shift) + 12ull * m.R;
+        const size_t smem = (32ull << m.shift) + fill_words(m.R) * 4;
         static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                             (32 << 12) + 12 * kMaxSplitRegions);
+                                                             (32 << 12) + fill_words(kMaxSplitRegions) * 4);
         const uint64_t part = std::max<uint64_t>(4 * (n / m.R + 1), 4ull << m.shift);
         const unsigned grid = static_cast<unsigned>(occupancy_smem(kern, kFillThreads, smem) * t->sm_count);
         e = attr != cudaSuccess ? attr

@@ -91,27 +91,41 @@ __global__ void __launch_bounds__(kPartThreads) k_part_hist(const K* __restrict_
   }
 }
 
-// Exclusive scan of cnt[0..R) by the whole block (R <= kMaxSplitRegions): give(r, before,
-// cnt[r]) is called once per region; ends with a barrier.  Up to 256 regions are scanned by
-// the first warp alone, 32 at a time, while the others wait (fewer instructions than every
-// warp's part of a block-wide scan).
-template <class Give>
-__device__ __forceinline__ void scan_regions(const uint32_t* cnt, uint32_t R, uint32_t* s_w, Give give) {
+// Words of shared memory that scan_regions takes for the counts and for their scan.
+__host__ __device__ constexpr uint32_t scan_cnt_words(uint32_t R) { return (R + 3) / 4 * 4; }
+__host__ __device__ constexpr uint32_t scan_off_words(uint32_t R) { return scan_cnt_words(R) + 4; }
+
+// Exclusive scan of cnt[0..R) into off[0..R], off[R] the total, by the whole block
+// (R <= kMaxSplitRegions; both 16-byte aligned, counts behind R up to scan_cnt_words are zero);
+// ends with a barrier.  Up to 512 regions are scanned by the first warp alone while the
+// others wait: a lane takes up to 16 neighbouring counts in 16-byte words, so the chain that
+// the block waits for is one scan over lanes.
+__device__ __forceinline__ void scan_regions(const uint32_t* cnt, uint32_t* off, uint32_t R, uint32_t* s_w) {
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (R <= 256) {
+  if (R <= 512) {
     if (warp == 0) {
-      uint32_t run = 0;
-      for (uint32_t r0 = 0; r0 < R; r0 += 32) {
-        const uint32_t c = r0 + lane < R ? cnt[r0 + lane] : 0u;
-        uint32_t inc = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(kFull, inc, o);
-          if (lane >= o) inc += y;
-        }
-        if (r0 + lane < R) give(r0 + lane, run + inc - c, c);
-        run += __shfl_sync(kFull, inc, 31);
+      const uint32_t b = lane * ((R + 127) / 128) * 4, end = min(b + (R + 127) / 128 * 4, scan_cnt_words(R));
+      uint32_t sum = 0;
+#pragma unroll 1
+      for (uint32_t i = b; i < end; i += 4) {
+        const uint4 v = *reinterpret_cast<const uint4*>(cnt + i);
+        sum += v.x + v.y + v.z + v.w;
       }
+      uint32_t inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+      }
+      uint32_t run = inc - sum;
+#pragma unroll 1
+      for (uint32_t i = b; i < end; i += 4) {  // the counts again: few registers held
+        const uint4 v = *reinterpret_cast<const uint4*>(cnt + i);
+        const uint4 o = make_uint4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
+        *reinterpret_cast<uint4*>(off + i) = o;
+        run = o.w + v.w;
+      }
+      if (lane == 31) off[R] = inc;  // what a word past the counts holds there already
     }
     __syncthreads();
     return;
@@ -138,8 +152,9 @@ __device__ __forceinline__ void scan_regions(const uint32_t* cnt, uint32_t R, ui
     if (w < warp) run += s_w[w];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
-    if (b0 + k < R) give(b0 + k, run, v[k]);
+    if (b0 + k < R) off[b0 + k] = run;
     run += v[k];
+    if (b0 + k == R - 1) off[R] = run;
   }
   __syncthreads();
 }
@@ -170,22 +185,29 @@ enum { kValsRead = 0, kValsLocal = 1, kValsNone = 2 };
 // region, then copy the runs out with consecutive threads on consecutive addresses.
 // Issue and the shared-memory pipe bound it (both about two thirds busy), so what an
 // element takes is kept short: its place in the output is delta[region] + its place in the
-// staged tile, position and region of a split with positions share one staged word, and the
-// scan over the regions is one warp's.  Pairs of at most 8 bytes come through a buffer that
-// cp.async fills for the next tile while this one is written out (no input is held in
-// registers, so three blocks fit an SM); wider ones are read into registers, two blocks.
-// One GB300, before -> now: 2^28 pairs of 8+4 bytes 1.94 -> 1.39 ms, 8+8 2.45 -> 2.17;
-// 2^27 queries of 4 bytes (with positions) 0.59 -> 0.49, 2^27 4+4-byte pairs 0.65 -> 0.66
-// (3.2 TB/s); 60 M keys alone 0.26 -> 0.19 (a set's 4-byte values of 1 are not written).
+// staged tile, position and region of a split with positions share one staged word.  What a
+// tile's barriers wait for is short too: the scan over the regions is one warp's and only
+// shared memory, the reservations (a global round trip) are made by all threads side by side.
+// 4-byte inputs come through buffers that cp.async fills for the next tile while this one is
+// written out (4-byte keys only if their values come that way too); 8-byte ones are read
+// into registers: through buffers 2^28 pairs of 8+8 bytes take 2.03 ms against 1.69, and
+// 8-byte keys beside buffered 4-byte values 1.80 against 1.49.  Pairs of at most 8 bytes hold
+// no input in registers and run three blocks an SM, wider ones two.
+// One GB300, with the reservations inside the one warp's scan -> as it is: 2^28 pairs of 8+8
+// bytes 2.09 -> 1.69 ms (5.1 TB/s), 8+4 1.85 -> 1.49, 2^28 queries of 8 bytes (with
+// positions) 1.66 -> 1.23, of 4 bytes 2^27 0.495 -> 0.473, 2^27 pairs of 4+4 0.662 -> 0.635,
+// 2^27 keys alone into 1300 regions 0.77 -> 0.59, 60 M into 256 0.188 -> 0.185.
 template <class K, class V, int kVals>
 struct SplitTile {
-  static constexpr bool kPre = sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) <= 8 && sizeof(K) == 4;
-  static constexpr int kMinBlocks = kPre ? 3 : 2;
-  // shared bytes of one element: staged key, value and region, input buffer
-  static constexpr size_t kElem = sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) + (kVals == kValsLocal ? 4 : 2) +
-                                  (kPre ? sizeof(K) + (kVals == kValsRead ? sizeof(V) : 0) : 0);
+  static constexpr bool kRead = kVals == kValsRead;
+  static constexpr bool kPreKey = sizeof(K) == 4 && (!kRead || sizeof(V) == 4);
+  static constexpr bool kPreVal = kRead && sizeof(V) == 4;
+  static constexpr int kMinBlocks = sizeof(K) + (kRead ? sizeof(V) : 0) <= 8 && sizeof(K) == 4 ? 3 : 2;
+  // shared bytes of one element: staged key, value and region, input buffers
+  static constexpr size_t kElem = sizeof(K) + (kRead ? sizeof(V) : 0) + (kVals == kValsLocal ? 4 : 2) +
+                                  (kPreKey ? sizeof(K) : 0) + (kPreVal ? sizeof(V) : 0);
   static constexpr size_t smem_bytes(uint32_t R, int tile) {
-    return kElem * tile + 4 * (4ull * R + kPartThreads / 32);
+    return kElem * tile + 4 * (2ull * scan_cnt_words(R) + 2ull * scan_off_words(R) + kPartThreads / 32);
   }
 };
 
@@ -196,7 +218,7 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
                    V* __restrict__ ovals, uint2* __restrict__ runs, const unsigned long long* n_dev) {
   if (n_dev != nullptr) n = *n_dev;
   using Tile = SplitTile<K, V, kVals>;
-  constexpr bool kPre = Tile::kPre, kRead = kVals == kValsRead;
+  constexpr bool kPreKey = Tile::kPreKey, kPreVal = Tile::kPreVal, kPre = kPreKey || kPreVal, kRead = Tile::kRead;
   constexpr int kTile = kPartThreads * kItems;
   extern __shared__ unsigned long long scatter_smem[];
   char* at = reinterpret_cast<char*>(scatter_smem);
@@ -210,14 +232,14 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
   uint2* s_pair = reinterpret_cast<uint2*>(at);
   K* s_key = reinterpret_cast<K*>(carve(sizeof(K) * kTile));
   V* s_val = reinterpret_cast<V*>(carve(kRead ? sizeof(V) * kTile : 0));
-  K* in_key = reinterpret_cast<K*>(carve(kPre ? sizeof(K) * kTile : 0));
-  V* in_val = reinterpret_cast<V*>(carve(kPre && kRead ? sizeof(V) * kTile : 0));
+  K* in_key = reinterpret_cast<K*>(carve(kPreKey ? sizeof(K) * kTile : 0));
+  V* in_val = reinterpret_cast<V*>(carve(kPreVal ? sizeof(V) * kTile : 0));
   using Reg = typename std::conditional<kVals == kValsLocal, uint32_t, uint16_t>::type;
   Reg* s_reg = reinterpret_cast<Reg*>(carve(sizeof(Reg) * kTile));  // region (<< 16 | position, with kValsLocal)
-  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(carve(4ull * m.R));
-  uint32_t* s_off = reinterpret_cast<uint32_t*>(carve(4ull * m.R));    // start in the staged tile
-  uint32_t* s_delta = reinterpret_cast<uint32_t*>(carve(4ull * m.R));  // output place - staged place
-  uint32_t* s_base = reinterpret_cast<uint32_t*>(carve(4ull * m.R));   // the region's start in the output
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(carve(4ull * scan_cnt_words(m.R)));
+  uint32_t* s_off = reinterpret_cast<uint32_t*>(carve(4ull * scan_off_words(m.R)));   // start in the staged tile
+  uint32_t* s_base = reinterpret_cast<uint32_t*>(carve(4ull * scan_off_words(m.R)));  // the region's start in the output
+  uint32_t* s_delta = reinterpret_cast<uint32_t*>(carve(4ull * scan_cnt_words(m.R)));  // output place - staged place
   uint32_t* s_w = reinterpret_cast<uint32_t*>(carve(4ull * (kPartThreads / 32)));
   const uint32_t nn = static_cast<uint32_t>(n);  // n < 2^32: places and counts are 32 bits
   const uint32_t ntiles = static_cast<uint32_t>((n + kTile - 1) / kTile);
@@ -226,32 +248,32 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
     const uint32_t b = tl * kTile;
     const uint32_t cnt = nn - b < kTile ? nn - b : kTile;
     for (uint32_t i = threadIdx.x; i < cnt; i += kPartThreads) {
-      cp_async_elem(in_key + i, keys + b + i);
-      if constexpr (kRead) cp_async_elem(in_val + i, vals + b + i);
+      if constexpr (kPreKey) cp_async_elem(in_key + i, keys + b + i);
+      if constexpr (kPreVal) cp_async_elem(in_val + i, vals + b + i);
     }
   };
   if constexpr (kPre) {
     if (blockIdx.x < ntiles) prefetch(blockIdx.x);
   }
   // region bases: exclusive prefix of the histogram (every block recomputes it)
-  for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) s_cnt[i] = hist[i];
+  for (uint32_t i = threadIdx.x; i < scan_cnt_words(m.R); i += kPartThreads) s_cnt[i] = i < m.R ? hist[i] : 0u;
   __syncthreads();
-  scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t) { s_base[r] = before; });
+  scan_regions(s_cnt, s_base, m.R, s_w);
   for (uint32_t i = threadIdx.x; i < m.R; i += kPartThreads) s_cnt[i] = 0;
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const uint32_t t0 = tile * kTile;
     const uint32_t tn = nn - t0 < kTile ? nn - t0 : kTile;
     if constexpr (kPre) cp_async_wait_all();  // this tile's input is in shared memory
     __syncthreads();
-    K kk[kPre ? 1 : kItems];
-    V vv[kPre || !kRead ? 1 : kItems];
+    K kk[kPreKey ? 1 : kItems];
+    V vv[kPreVal || !kRead ? 1 : kItems];
     uint32_t rr[kItems];  // region << 16 | rank (a tile holds fewer than 2^16 elements)
-    if constexpr (!kPre) {
+    if constexpr (!kPreKey || (kRead && !kPreVal)) {
 #pragma unroll
       for (int k = 0; k < kItems; ++k) {
         const uint32_t i = k * kPartThreads + threadIdx.x;
-        kk[k] = i < tn ? ldg_stream(keys + t0 + i) : K(0);
-        if constexpr (kRead) vv[k] = i < tn ? ldg_stream(vals + t0 + i) : V(0);
+        if constexpr (!kPreKey) kk[k] = i < tn ? ldg_stream(keys + t0 + i) : K(0);
+        if constexpr (kRead && !kPreVal) vv[k] = i < tn ? ldg_stream(vals + t0 + i) : V(0);
       }
     }
 #pragma unroll
@@ -259,18 +281,19 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
       const uint32_t i = k * kPartThreads + threadIdx.x;
       if (i < tn) {
         uint32_t r;
-        if constexpr (kPre) r = m.of(in_key[i]);
+        if constexpr (kPreKey) r = m.of(in_key[i]);
         else r = m.of(kk[k]);
         rr[k] = r << 16 | atomicAdd(s_cnt + r, 1u);
       }
     }
     __syncthreads();
-    scan_regions(s_cnt, m.R, s_w, [&](uint32_t r, uint32_t before, uint32_t c) {
+    scan_regions(s_cnt, s_off, m.R, s_w);
+    for (uint32_t r = threadIdx.x; r < m.R; r += kPartThreads) {
+      const uint32_t before = s_off[r], c = s_cnt[r];
       const uint32_t p = c ? s_base[r] + atomicAdd(cursor + r, c) : 0u;
-      s_off[r] = before;
       s_delta[r] = p - before;
       if constexpr (kVals == kValsLocal) runs[static_cast<uint64_t>(tile) * m.R + r] = make_uint2(p, before);
-    });
+    }
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
       const uint32_t i = k * kPartThreads + threadIdx.x;
@@ -279,9 +302,10 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
         if constexpr (kPair) {
           s_pair[o] = make_uint2(in_key[i], in_val[i]);
         } else {
-          if constexpr (kPre) s_key[o] = in_key[i];
+          if constexpr (kPreKey) s_key[o] = in_key[i];
           else s_key[o] = kk[k];
-          if constexpr (kRead) s_val[o] = vv[k];
+          if constexpr (kPreVal) s_val[o] = in_val[i];
+          else if constexpr (kRead) s_val[o] = vv[k];
         }
         if constexpr (kVals == kValsLocal) s_reg[o] = r << 16 | i;
         else s_reg[o] = static_cast<Reg>(r);
