@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kExecThreads, 3) k_exec(const ExecHeader* __re
         sv_erase_range<L, GR, SR>(t, keys, src, flags, removed, none);
         delta = -removed;
       } else if constexpr (kOne) {  // positions inside the tile, buffers from its start
-        BatchBlocks blocks(static_cast<uint32_t>(end - begin));
+        BatchBlocks<false> blocks(static_cast<uint32_t>(end - begin));
         Queue& q = s_q[threadIdx.x >> 5];
         if (op == WC_OP_INSERT) {
           insert_blocks<L, W>(t, keys + begin, vals + begin, blocks, q.put, flags, delta);

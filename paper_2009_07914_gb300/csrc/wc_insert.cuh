@@ -11,8 +11,8 @@
 // or its end.
 //
 // The sweep of 2^27 pairs, one GB300, that engine against this kernel (with half-line
-// reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.86 ms, at 0.5 3.11 -> 2.30;
-// 8+8 bytes at 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.  In input order, 2^20
+// reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.86 ms (2.63 with the table
+// copied to L2 ahead of the sweep, BatchBlocks::prefetch), at 0.5 3.11 -> 2.30; 8+8 bytes at 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.  In input order, 2^20
 // pairs at 0.9 65.7 -> 65.6 us, at 0.5 44.0 -> 40.1; half a table erased and inserted again
 // (2^20 keys, 0.9) 172 -> 118 us.
 #pragma once
@@ -102,9 +102,9 @@ struct InsertQueue {
 
 // The inserts of a warp's blocks; every lane calls.  vals == nullptr: every value is 1 (sets;
 // counting tables without weights).  added: new keys stored by this lane.
-template <class L, int W>
+template <class L, int W, bool kSwept>
 __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename L::Key* __restrict__ keys,
-                                              const typename L::Val* __restrict__ vals, BatchBlocks& blocks,
+                                              const typename L::Val* __restrict__ vals, BatchBlocks<kSwept>& blocks,
                                               InsertQueue<typename L::Key, typename L::Val>& q, uint32_t& flags,
                                               long long& added) {
   using Slot = typename L::Slot;
@@ -233,9 +233,9 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
   while (cnt > 0) drain();
 }
 
-// counter != nullptr: a batch split by table region, swept in order.  n_dev (or null): the
+// kSwept: a batch split by table region, swept in order by `counter`.  n_dev (or null): the
 // batch's size on the device, at most n.
-template <class L, int W>
+template <class L, int W, bool kSwept>
 __global__ void __launch_bounds__(kLookThreads, 4)
     k_insert(TableDesc t, const typename L::Key* __restrict__ keys, const typename L::Val* __restrict__ vals,
              uint64_t n, unsigned long long* counter, const unsigned long long* n_dev) {
@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(kLookThreads, 4)
   __shared__ InsertQueue<typename L::Key, typename L::Val> q[kLookThreads / 32];
   uint32_t flags = 0;
   long long added = 0;
-  BatchBlocks blocks(n, counter);
+  BatchBlocks<kSwept> blocks(n, counter, 512, false);
+  blocks.prefetch(t.slots, static_cast<uint64_t>(t.p) * W * slot_size<L>());
   insert_blocks<L, W>(t, keys, vals, blocks, q[threadIdx.x >> 5], flags, added);
   flush_flags(t.status, flags);
   flush_delta(t.size, added);
@@ -262,7 +263,7 @@ inline int insert_blocks_per_sm(const wc_table* t, int most, uint64_t n, bool sw
 template <class L, int W>
 cudaError_t insert_launch(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
                           unsigned long long* counter, const unsigned long long* n_dev, cudaStream_t s) {
-  auto kern = k_insert<L, W>;
+  auto kern = counter != nullptr ? k_insert<L, W, true> : k_insert<L, W, false>;
   const int per_sm = insert_blocks_per_sm(t, occupancy(kern, kLookThreads), n, counter != nullptr);
   const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
   const uint64_t most = static_cast<uint64_t>(per_sm) * t->sm_count;

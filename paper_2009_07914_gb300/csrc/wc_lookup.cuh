@@ -24,7 +24,8 @@
 namespace wc {
 
 constexpr int kLookThreads = 256;
-constexpr uint32_t kLookChunk = 512;  // queries a warp takes from the sweep counter at a time
+constexpr uint32_t kLookChunk = 512;  // keys a warp of the group-per-key engine takes from the sweep counter at a time
+constexpr uint64_t kSweepLead = 8ull << 20;  // table bytes a sweep's prefetch runs ahead (BatchBlocks::prefetch)
 
 template <class L>
 constexpr int slot_size() {
@@ -134,32 +135,87 @@ __device__ __forceinline__ Probe<L> probe_window(const typename L::Slot* slots, 
   return r;
 }
 
-// A warp's blocks of 32 consecutive inputs (warp-uniform).  counter != nullptr: chunks of
-// kLookChunk inputs are taken from it in order, so the grid sweeps the batch front to back;
-// otherwise the blocks are strided over the grid.  Inputs are numbered in 32 bits (n < 2^32).
+// Regions that a batch of queries is split into (MiB), and the inputs of a chunk of its
+// sweep.  Small ones sweep faster: 2^27 queries of 4+4 bytes over 1.2 GiB in regions of 32
+// MiB and chunks of 512 1.67 ms, 16 and 512 1.52, 16 and 256 1.45 (32 and 256 1.60); 8 MiB
+// 1.49.  Twice the regions split and put back slower (0.04 ms there), which large tables
+// do not get back: 2^28 Zipf queries of 8+8 bytes over 4.8 GiB sweep in 2.89 ms with 32 and
+// 512 (3.07 with 256) and 2.84 with 16, for 0.6 ms more before and after.
+constexpr uint64_t kSmallSweep = 2ull << 30;
+__host__ __device__ constexpr int look_region_mib(uint64_t table_bytes) { return table_bytes > kSmallSweep ? 32 : 16; }
+__host__ __device__ constexpr uint32_t look_chunk(uint64_t table_bytes) { return table_bytes > kSmallSweep ? 512 : 256; }
+
+// A warp's blocks of 32 consecutive inputs (warp-uniform).  kSwept: chunks of inputs are taken
+// from a counter in order, so the grid sweeps the batch front to back; otherwise the blocks
+// are strided over the grid (kernels of their own: a direct batch carries none of the sweep's
+// registers).  Inputs are numbered in 32 bits (n < 2^32).
+//
+// What the warps of a sweep hold together is the part of the table that has to stay in L2,
+// so chunks are short, and a sweep of lookups asks for the next one when one is begun
+// (early), so no warp waits for the counter.  Chunks of 192, 128 and 64: 1.47, 1.65 and 2.9
+// ms for 2^27 lookups, as the counter takes only some 0.3 to 0.7 atomics per ns.  It takes
+// fewest beside inserts, which are fastest with 512 asked for when needed (2^27 pairs of 4+4
+// bytes 2.63 ms, early 2.84, early 256 2.78; 2^26 Zipf counting inserts 0.63, early 256
+// 0.88).  Batches below 2^21 take shorter chunks: there are about 5000 warps.
+template <bool kSwept>
 struct BatchBlocks {
   uint32_t n, next, end;  // end of the taken chunk
-  uint32_t stride;
+  uint32_t stride;        // between a warp's blocks; of a sweep, inputs of a chunk
   unsigned long long* counter;
-  __device__ __forceinline__ BatchBlocks(uint64_t n_, unsigned long long* c)
-      : n(static_cast<uint32_t>(n_)), next(c != nullptr ? n : (blockIdx.x * blockDim.x + threadIdx.x) & ~31u), end(n),
-        stride(gridDim.x * blockDim.x), counter(c) {}
+  unsigned long long later;  // first input of the chunk after this one (lane 0)
+  const char* tab = nullptr;  // prefetch: the table, its bytes, bytes per input << 16
+  uint64_t tab_bytes = 0, ratio = 0;
+  bool early;  // ask for the next chunk when one is begun
+  // most: inputs of a chunk
+  __device__ __forceinline__ BatchBlocks(uint64_t n_, unsigned long long* c, uint32_t most, bool early_)
+      : n(static_cast<uint32_t>(n_)), next(kSwept ? n : (blockIdx.x * blockDim.x + threadIdx.x) & ~31u), end(n),
+        stride(kSwept ? min(most, max(32u, n >> 12 & ~31u)) : gridDim.x * blockDim.x), counter(c), later(0),
+        early(early_) {
+    if (kSwept && early) ask();
+  }
   // all of n inputs for this warp (one tile of the batched executor)
-  __device__ __forceinline__ explicit BatchBlocks(uint32_t n_) : n(n_), next(0), end(n_), stride(32), counter(nullptr) {}
+  __device__ __forceinline__ explicit BatchBlocks(uint32_t n_)
+      : n(n_), next(0), end(n_), stride(32), counter(nullptr), later(0), early(false) {}
+  __device__ __forceinline__ void ask() {
+    if ((threadIdx.x & 31) == 0) later = atomicAdd(counter, static_cast<unsigned long long>(stride));
+  }
+  // A sweep of inserts copies the table to L2 kSweepLead ahead of itself, in order, as much
+  // per chunk as its share of the batch: the windows it reads next are not fetched one by one
+  // from DRAM.  A batch that would not touch most windows is left alone; for a skewed one the
+  // place in the table is a guess and the copies are at most the table's size.
+  // 2^27 pairs of 4+4 bytes 2.97 -> 2.74 ms, 2^28 of 8+8 8.19 -> 7.94 (16 MiB ahead 2.76 and
+  // 8.15), counting and set inserts 2 and 1 %.  Lookups gain nothing (1.46 ms both ways,
+  // 8-byte ones 2.94 -> 3.1), inserts of open-addressing multi-value tables lose (2^26 1.81
+  // -> 1.91): neither calls this.
+  __device__ __forceinline__ void prefetch(const void* slots, uint64_t bytes) {
+    if (!kSwept || bytes > static_cast<uint64_t>(n) * 64) return;
+    tab = static_cast<const char*>(slots);
+    tab_bytes = bytes & ~127ull;
+    ratio = (bytes << 16) / n;  // n > 0: a table has bytes
+  }
+  __device__ __forceinline__ void prefetch_for(uint64_t c) const {
+    const uint64_t a = (c * ratio >> 16 & ~127ull) + kSweepLead;
+    uint64_t e = ((c + stride) * ratio >> 16 & ~127ull) + kSweepLead;
+    if (e > tab_bytes) e = tab_bytes;
+    if (a < e)  // at most 16 KiB
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(tab + a), "r"(static_cast<uint32_t>(e - a))
+                   : "memory");
+  }
   // first input of the next block, n when there is none
   __device__ __forceinline__ uint32_t take() {
-    if (counter == nullptr) {
+    if constexpr (!kSwept) {
       const uint32_t b = next;
       next = b < n && n - b > stride ? b + stride : n;
       return b < n ? b : n;
     }
     if (next >= end) {
-      unsigned long long c = 0;
-      if ((threadIdx.x & 31) == 0) c = atomicAdd(counter, static_cast<unsigned long long>(kLookChunk));
-      c = __shfl_sync(kFull, c, 0);
-      if (c >= n) return n;  // and so every time from now on: the counter only grows
+      if (!early) ask();
+      const unsigned long long c = __shfl_sync(kFull, later, 0);
+      if (c >= n) return n;  // and so every time from now on
+      if (early) ask();
+      if (tab != nullptr && (threadIdx.x & 31) == 0) prefetch_for(c);
       next = static_cast<uint32_t>(c);
-      end = n - next > kLookChunk ? next + kLookChunk : n;
+      end = n - next > stride ? next + stride : n;
     }
     const uint32_t b = next;
     next = end - b > 32 ? b + 32 : end;
@@ -176,8 +232,8 @@ struct LookupQueue {
 };
 
 // The lookups of a warp's blocks; every lane calls.
-template <class L, int W, class Emit, class KIn>
-__device__ __forceinline__ void lookup_blocks(const TableDesc& t, const KIn* __restrict__ keys, BatchBlocks& blocks,
+template <class L, int W, bool kSwept, class Emit, class KIn>
+__device__ __forceinline__ void lookup_blocks(const TableDesc& t, const KIn* __restrict__ keys, BatchBlocks<kSwept>& blocks,
                                               LookupQueue<KIn>& q, const Emit& emit, uint32_t& flags) {
   using Slot = typename L::Slot;
   using Key = typename L::Key;
@@ -257,20 +313,21 @@ __device__ __forceinline__ void lookup_blocks(const TableDesc& t, const KIn* __r
   while (cnt > 0) drain();
 }
 
-// counter != nullptr: a batch sorted by table region, swept in order.
-template <class L, int W, class Emit, class KIn = typename L::Key>
+// kSwept: a batch sorted by table region, swept in order by `counter`.
+template <class L, int W, class Emit, class KIn, bool kSwept>
 __global__ void __launch_bounds__(kLookThreads, 5) k_lookup(TableDesc t, const KIn* __restrict__ keys, uint64_t n,
                                                             unsigned long long* counter, Emit emit) {
   __shared__ LookupQueue<KIn> q[kLookThreads / 32];
   uint32_t flags = 0;
-  BatchBlocks blocks(n, counter);
+  const uint64_t bytes = static_cast<uint64_t>(t.p) * W * slot_size<L>();
+  BatchBlocks<kSwept> blocks(n, counter, look_chunk(bytes), true);
   lookup_blocks<L, W>(t, keys, blocks, q[threadIdx.x >> 5], emit, flags);
   flush_flags(t.status, flags);
 }
 
 // Lookups of a batch split by region (the blocked scheme) sweep the table region by region
 // in L2: 2^27 queries of 4+4-byte pairs over a 1.1 GiB table take 0.20 ms to count the
-// regions, 0.59 ms to split, 1.68 ms to probe and 0.41 ms to put back, against 4.71 ms in
+// regions, 0.48 ms to split, 1.45 ms to probe and 0.44 ms to put back, against 4.71 ms in
 // input order (5.14 on the group-per-key engine).
 //
 // Results of a batch split by region, back in input order: the split kept every input
@@ -359,7 +416,7 @@ __global__ void __launch_bounds__(kPartThreads, 3) k_unsplit(const uint16_t* __r
 template <class L, int W, class Emit, class KIn = typename L::Key>
 cudaError_t lookup_launch(const wc_table* t, const KIn* keys, uint64_t n, unsigned long long* counter,
                           const Emit& emit, cudaStream_t s) {
-  auto kern = k_lookup<L, W, Emit, KIn>;
+  auto kern = counter != nullptr ? k_lookup<L, W, Emit, KIn, true> : k_lookup<L, W, Emit, KIn, false>;
   const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
   const uint64_t most = static_cast<uint64_t>(occupancy(kern, kLookThreads)) * t->sm_count;
   return launch_k(t, kern, static_cast<unsigned>(std::min(want, most)), kLookThreads, 0, s, desc_of(t), keys, n,
@@ -379,7 +436,7 @@ struct QuerySplit {
 template <class K, class V>
 cudaError_t query_split(const wc_table* t, int region_mib, const K* keys, uint64_t n, cudaStream_t s,
                         QuerySplit<K, V>& q) {
-  const RegionMap m = region_map(t, region_mib);
+  const RegionMap m = region_map(t, region_mib > 0 ? region_mib : look_region_mib(t->table_bytes));
   q.R = m.R;
   const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
   const uint64_t rv_bytes = align256(n * sizeof(V)), rf_bytes = align256(n);

@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kLookThreads, 4)
   Slot* slots = static_cast<Slot*>(t.slots);
   uint32_t flags = 0, cnt = 0;
   long long added = 0;
-  BatchBlocks blocks(n, counter);
+  BatchBlocks<true> blocks(n, counter, 512, false);
 
   struct Pair {
     Key k;
@@ -427,7 +427,8 @@ __global__ void __launch_bounds__(kLookThreads, 5)
   const uint32_t below = (1u << lane) - 1u;
   const Slot* slots = static_cast<const Slot*>(t.slots);
   uint32_t flags = 0, cnt = 0;
-  BatchBlocks blocks(n, counter);
+  BatchBlocks<std::is_same<Out, uint32_t>::value> blocks(  // 32-bit counts: of a batch split by region
+      n, counter, look_chunk(static_cast<uint64_t>(t.p) * W * slot_size<L>()), true);
 
   struct Query {
     Key k;

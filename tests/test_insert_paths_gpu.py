@@ -98,3 +98,19 @@ def test_last_slots_and_repeats(wc, kb, W):
     assert big.insert(k, v) == wc.WC_FLAG_DUPLICATE_KEY and big.size() == 997
     out, found, _ = big.retrieve(k[:997])
     assert found.all() and np.array_equal(out.astype(np.int64) % 997, pick[:997])
+
+
+@pytest.mark.parametrize("kb,n,load", [(4, (1 << 19) + 13, 0.9), (4, (1 << 21) + 5, 0.9), (8, (1 << 22) + 77, 0.9),
+                                       (4, (1 << 19) + 31, 0.05), (8, (1 << 18) + 1, 0.005)])
+def test_sweeps_of_every_chunk_length(wc, kb, n, load):
+    """Chunks of 32 to 256 inputs; tables that end inside the prefetched range, in front of
+    it, or are so large beside the batch that nothing is prefetched."""
+    keys, vals = _inputs(kb, n, n)
+    t = wc.SingleValueTable(kb, kb, min_capacity=int(n / load) + 1, seed=SEED)
+    for op in (wc.WC_OP_INSERT, wc.WC_OP_RETRIEVE):
+        lc = wc.wc_table_get_launch(t.handle, op)
+        t.set_launch(op, lc["group_size"], scheme=wc.WC_SCHEME_BLOCKED, region_mib=1)
+    assert t.insert(keys, vals) == 0 and t.size() == n
+    out, found, _ = t.retrieve(keys)
+    assert found.all()
+    np.testing.assert_array_equal(out, vals)
