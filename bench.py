@@ -103,7 +103,7 @@ def peaks():
 # Sources of the single-value probe kernels (a change to any of them invalidates the
 # committed traffic record of those kernels).
 SV_KERNEL_SOURCES = ("wc_device.cuh", "wc_sv_kernels.cuh", "wc_sv_dispatch.cuh", "wc_partition.cuh",
-                     "wc_launch.cuh", "wc_sv_p32.cu")
+                     "wc_launch.cuh", "wc_lookup.cuh", "wc_insert.cuh", "wc_sv_p32.cu")
 
 
 def _code_only(text: str) -> str:
@@ -497,7 +497,11 @@ def run_wc(args, rank, world, local_rank):
     achieved = BYTES_PER_OP[dom] * n / (dom_ms * 1e-3) / 1e9
     workload_name = "sv_u32_n2^%d_alpha%.2f" % (args.log2n, args.alpha)
     kif_ret = api.wc_table_get_launch(h, wc.WC_OP_RETRIEVE)["keys_in_flight"]
-    kname = "k_sv_insert" if dom == "insert" else ("k_sv_retrieve2" if kif_ret == 2 else "k_sv_retrieve")
+    narrow = info["window_width"] * info["slot_bytes"] <= 64  # one key per thread
+    if dom == "insert":
+        kname = "k_insert" if narrow else "k_sv_insert"
+    else:
+        kname = "k_lookup" if narrow else "k_sv_retrieve2" if kif_ret == 2 else "k_sv_retrieve"
     traffic = ncu_traffic(kname, workload_name)
     cpu = None if args.no_cpu else cpu_baseline(23, args.alpha)
     res = {
@@ -735,7 +739,9 @@ def run_sv64_zipf(args, dev):
             (insert_launches(api, h, n) + lookup_launches(api, h, n)) * args.steps,
             {"insert_gops": n / ins / 1e6, "retrieve_gops": n / ret / 1e6, "insert_ms": ins, "retrieve_ms": ret,
              "retrieve_dedup_gops": n / ret_dedup / 1e6, "retrieve_dedup_ms": ret_dedup,
-             "roofline": {"bound": "hbm", "kernel": "k_sv_retrieve", "achieved": 48 * n / (ret * 1e-3) / 1e9,
+             "roofline": {"bound": "hbm",
+                          "kernel": "k_lookup" if info["window_width"] * info["slot_bytes"] <= 64 else "k_sv_retrieve",
+                          "achieved": 48 * n / (ret * 1e-3) / 1e9,
                           "peak": peak, "unit": "GB/s", "frac": 48 * n / (ret * 1e-3) / 1e9 / peak,
                           "bytes_per_op": 48, "traffic": None}})
     api.wc_table_destroy(h)
