@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) k_bloom_insert(TableDesc t, const K* __re
 // keys (a skewed batch) is worked on in parts of at most `part` keys, each with a copy of
 // its own, so no block is left with a hot key's share.  Concurrent inserts stay correct:
 // the filter only ever changes by ORs.  2^27 keys of a 160 MiB filter, k = 7: 0.93 ms (1.60
-// with 512 threads: one block of a 128 KiB region fills an SM), 1.91 ms with the split,
+// with 512 threads: one block of a 128 KiB region fills an SM), 1.73 ms with the split,
 // against 3.89 ms by k_bloom_insert and 6.65 ms with its former 32-bit words.
 constexpr int kFillThreads = 1024;
 constexpr uint32_t fill_words(uint32_t R) { return scan_cnt_words(R) + 2 * scan_off_words(R); }
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256) k_bloom_contains(TableDesc t, const K* __
 
 // Inserts are split where the shared-memory copies save more global atomics than merging
 // them takes: k = 7, 10 bits per key, in input order against split, 2^22 keys 79.8 / 119.7
-// us, 2^24 287 / 278, 2^26 (80 MiB) 1164 / 976, 2^27 (160 MiB) 3892 / 1909.  A copy is merged
+// us, 2^24 287 / 278, 2^26 (80 MiB) 1164 / 976, 2^27 (160 MiB) 3892 / 1730.  A copy is merged
 // whatever the batch, so a batch below a quarter key per byte of the filter stays in order.
 // Filters of more regions than a split takes (above 256 MiB) are swept by k_bloom_insert
 // over a split into L2-sized regions (2^28 keys, 320 MiB: 11.7 ms in input order).

@@ -44,7 +44,8 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
     // About 128 regions rather than L2-sized ones: a tile of one region then holds fewer
     // distinct keys (2^28 Zipf inserts over 2^24 keys: 26 % of a tile's elements in 160
     // regions, 44 % in 11), and each costs a probe and two atomics.  Insert 8.71 -> 7.93 ms,
-    // the split itself 1.4 -> 1.85 of it.
+    // the split itself 1.4 -> 1.85 of it (1.86 with its
+    // histogram now, of 7.3 ms).
     const uint64_t mib = std::min<uint64_t>(32, std::max<uint64_t>(1, t->table_bytes >> 27));
     e = region_split(t, region_map(t, static_cast<int>(mib)), k, static_cast<const V*>(vals), n, s, sp, rec_bytes);
     if (e != cudaSuccess) return e;
