@@ -70,8 +70,10 @@ enum {
  *                       slot of the single-value slot layouts along the key's probing
  *                       sequence (Sec. IV and Sec. V-C, the multi-value hash table).  Insert
  *                       appends; count_values / retrieve_multi walk the sequence up to the
- *                       first window holding an empty slot and count or copy every match;
- *                       erase tombstones every copy.  wc_retrieve is not available.
+ *                       first window holding an empty slot -- or one that no copy of a key
+ *                       with the query's tag walked past (one byte per window beside the
+ *                       slots; snapshots leave it out) -- and count or copy every match; erase
+ *                       tombstones every copy.  wc_retrieve is not available.
  *   WC_HASH_SET         a set of keys (Sec. IV: HashSet), one 4- or 8-byte key per slot
  *                       (value_bytes 0): insert, wc_contains, erase.
  *   WC_COUNTING         occurrence counts per key (Sec. IV: CountingHashTable), the
@@ -221,7 +223,8 @@ typedef struct {
  * counting, hash-set and open-addressing multi-value tables; retrieves of single-value and
  * counting tables (the results are put back in input order).  WC_SCHEME_AUTO picks
  * BLOCKED for those inserts when the batch holds at least 2^18 pairs and the table is
- * larger than 64 MiB, for lookups (wc_retrieve, wc_contains; hash sets too) when the slots
+ * larger than 64 MiB, for lookups (wc_retrieve, wc_contains; hash sets too; and the counts of
+ * multi-value tables with windows of at most 64 bytes) when the slots
  * take more than 512 MiB and the batch holds at least one query per 64 bytes of them (and
  * the stream is not being captured and the scratch fits), DIRECT otherwise.
  * WC_SCHEME_DEDUP (lookups of single-value, counting and hash-set tables: wc_retrieve,
