@@ -105,7 +105,11 @@ __global__ void __launch_bounds__(256) k_bloom_insert(TableDesc t, const K* __re
 // the filter only ever changes by ORs.  2^27 keys of a 160 MiB filter, k = 7: 0.93 ms (1.60
 // with 512 threads: one block of a 128 KiB region fills an SM), 1.73 ms with the split,
 // against 3.89 ms by k_bloom_insert and 6.65 ms with its former 32-bit words.
+// A part is at most kFillPart keys, so its size and the parts' number stay far below 2^32
+// for any batch, and a filter of one region is still filled by many blocks (the unit words
+// are 32 bits wide; a batch has up to 2^32 - 1 keys).
 constexpr int kFillThreads = 1024;
+constexpr uint64_t kFillPart = 1ull << 20;
 constexpr uint32_t fill_words(uint32_t R) { return scan_cnt_words(R) + 2 * scan_off_words(R); }
 
 template <class K>
@@ -123,7 +127,8 @@ __global__ void __launch_bounds__(kFillThreads) k_bloom_fill(TableDesc t, const 
   for (uint32_t r = threadIdx.x; r < scan_cnt_words(m.R); r += kFillThreads) s_cnt[r] = r < m.R ? hist[r] : 0u;
   __syncthreads();
   scan_regions(s_cnt, s_off, m.R, s_w);
-  for (uint32_t r = threadIdx.x; r < m.R; r += kFillThreads) s_cnt[r] = (s_cnt[r] + part - 1) / part;
+  for (uint32_t r = threadIdx.x; r < m.R; r += kFillThreads)
+    if (s_cnt[r] != 0) s_cnt[r] = (s_cnt[r] - 1) / part + 1;
   __syncthreads();
   scan_regions(s_cnt, s_unit, m.R, s_w);
   const uint32_t units = s_unit[m.R];
@@ -230,7 +235,7 @@ cudaError_t insert(const wc_table* t, const K* keys, uint64_t n, cudaStream_t s)
         const size_t smem = (32ull << m.shift) + fill_words(m.R) * 4;
         static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                              (32 << 12) + fill_words(kMaxSplitRegions) * 4);
-        const uint64_t part = std::max<uint64_t>(4 * (n / m.R + 1), 4ull << m.shift);
+        const uint64_t part = std::min(std::max<uint64_t>(4 * (n / m.R + 1), 4ull << m.shift), kFillPart);
         const unsigned grid = static_cast<unsigned>(occupancy_smem(kern, kFillThreads, smem) * t->sm_count);
         e = attr != cudaSuccess ? attr
                                 : launch_k(t, kern, grid, kFillThreads, smem, s, desc_of(t), sp.keys, m, sp.hist,

@@ -51,3 +51,24 @@ def test_split_batches_equal_small_ones(wc, kb, bits, k):
     assert torch.equal(fa, fb)
     real = (q[::2] != 0) & (q[::2] != -1)
     assert (fa[::2][real] == 1).all()
+
+
+@pytest.mark.parametrize("blocks,n", [(31, 900_000_000), (31, (1 << 30) - 1), (64, 1_700_000_000)])
+def test_large_batches_into_small_filters(wc, blocks, n):
+    """Hundreds of millions of keys of one or two regions (part sizes and unit counts past
+    32 bits if they grew with the batch): the same bits and size as a few keys at a time."""
+    import torch
+    from paper_2009_07914_gb300 import api
+    a, b = (wc.BloomFilterTable(4, bits=256 * blocks, k=7) for _ in range(2))
+    few = torch.arange(1, 129, device="cuda", dtype=torch.int32) * 7919
+    keys = few[:3].repeat((n + 2) // 3)[:n].contiguous()  # three keys again and again, then all of them
+    keys[-128:] = few
+    api.wc_insert(a.handle, keys, None)
+    api.wc_insert(b.handle, few, None)
+    assert a.size() == n and b.size() == 128
+    assert a.status(clear=True) == b.status(clear=True) == 0
+    da, db = api.wc_table_dump_slots(a.handle), api.wc_table_dump_slots(b.handle)
+    assert np.array_equal(da, db) and da.any()
+    f = torch.zeros(128, dtype=torch.uint8, device="cuda")
+    api.wc_contains(a.handle, few, f)
+    assert bool((f == 1).all())
