@@ -46,12 +46,11 @@ __device__ __forceinline__ uint32_t spot_word(const typename L::Slot (&s)[S], ty
   return hit | tomb | used;
 }
 
-// Window w seen by the key k in every lane with `on`; every lane of the warp calls.  As in
+// Window w seen by the key k; every lane of the warp calls, with a window of the table.  As in
 // probe_window, a pair of lanes reads a 64-byte window in one request.
 template <class L, int W>
-__device__ __forceinline__ Spot spot_of(const typename L::Slot* slots, bool on, typename L::Key k, uint32_t w) {
+__device__ __forceinline__ Spot spot_of(const typename L::Slot* slots, typename L::Key k, uint32_t w) {
   using Slot = typename L::Slot;
-  w = on ? w : 0u;  // a lane without a key reads the first window
   uint32_t lo, hi = 0;  // the window's first half (or all of it), its second
   if constexpr (W * slot_size<L>() <= 32) {
     Slot s[W];
@@ -130,7 +129,7 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
   // slot is taken to hold the word that clears and erases leave; a pair that has lost a slot
   // reads the word again before its CAS.
   auto step = [&](bool& on, Pair& x) {
-    const Spot s = spot_of<L, W>(slots, on, x.k, x.w);
+    const Spot s = spot_of<L, W>(slots, x.k, x.w);
     if (!on) return;
     const uint64_t base = static_cast<uint64_t>(x.w) * W;
     if (s.hit) {  // overwrite the value (duplicate warning, Sec. IV-B3)
@@ -203,6 +202,7 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
       x.tomb = q.tomb[cnt + lane];
     }
     __syncwarp();
+    x.w = window_for_all(on, x.w);
     x.h = fmix64(static_cast<uint64_t>(x.k) ^ t.seed);
     step(on, x);
     enqueue(on, x);

@@ -265,11 +265,10 @@ __device__ __forceinline__ uint32_t oa_word(const typename L::Slot (&s)[S], type
   return kCountKey ? m : m << first;
 }
 
-// The same of window w for the lanes with `on`; every lane of the warp calls.
+// The same of window w; every lane of the warp calls, with a window of the table.
 template <class L, int W, bool kCountKey>
-__device__ __forceinline__ uint32_t oa_window(const typename L::Slot* slots, bool on, typename L::Key k, uint32_t w) {
+__device__ __forceinline__ uint32_t oa_window(const typename L::Slot* slots, typename L::Key k, uint32_t w) {
   using Slot = typename L::Slot;
-  w = on ? w : 0u;
   if constexpr (W * slot_size<L>() <= 32) {
     Slot s[W];
     load_slots<L, W, !kCountKey>(slots + static_cast<uint64_t>(w) * W, s);
@@ -322,7 +321,7 @@ __global__ void __launch_bounds__(kLookThreads, 4)
     uint64_t h;
   };
   auto step = [&](bool& on, Pair& x) {
-    const uint32_t m = oa_window<L, W, false>(slots, on, x.k, x.w);
+    const uint32_t m = oa_window<L, W, false>(slots, x.k, x.w);
     if (!on) return;
     const uint32_t fr = m & 0xffffu;
     if (fr == 0) {
@@ -379,6 +378,7 @@ __global__ void __launch_bounds__(kLookThreads, 4)
       x.salt = q.salt[cnt + lane];
     }
     __syncwarp();
+    x.w = window_for_all(on, x.w);
     x.h = fmix64(static_cast<uint64_t>(x.k) ^ t.seed);
     step(on, x);
     enqueue(on, x);
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kLookThreads, 5)
     uint64_t h;
   };
   auto step = [&](bool& on, Query& x) {
-    const uint32_t m = oa_window<L, W, true>(slots, on, x.k, x.w);
+    const uint32_t m = oa_window<L, W, true>(slots, x.k, x.w);
     if (!on) return;
     x.cnt += m >> 24;
     bool more = (m & 0xffffu) == 0;  // no empty slot
@@ -474,6 +474,7 @@ __global__ void __launch_bounds__(kLookThreads, 5)
       x.cnt = q.cnt[cnt + lane];
     }
     __syncwarp();
+    x.w = window_for_all(on, x.w);
     x.h = fmix64(static_cast<uint64_t>(x.k) ^ t.seed);
     step(on, x);
     enqueue(on, x);

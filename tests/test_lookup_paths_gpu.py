@@ -127,3 +127,44 @@ def test_lookup_in_a_graph_keeps_no_scratch(wc):
             torch.cuda.synchronize()
         np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), eo)
         np.testing.assert_array_equal(found.cpu().numpy(), ef)
+
+
+def _graph_us(f, reps):
+    import torch
+    f()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(reps):
+            f()
+    best = float("inf")
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        g.replay()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / reps * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("kb,W", [(4, 8), (8, 4)])
+def test_tails_of_many_warps_do_not_meet_on_one_line(wc, kb, W):
+    """Lookups of batches that give a warp about one block of queries are as long as their
+    longest walks: 300,000 queries take less than twice as long as 70,000 (about 1.45 times;
+    2.2 to 2.5 times when lanes without a query all read the table's first window)."""
+    import torch
+    from paper_2009_07914_gb300 import api
+    us = []
+    for n in (70_000, 300_000):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(n)
+        span = (1, 2 ** 31 - 1) if kb == 4 else (1, 2 ** 62)
+        keys = torch.randint(*span, (2 * n,), generator=g, device="cuda", dtype=torch.int32 if kb == 4 else torch.int64)
+        t = wc.SingleValueTable(kb, kb, min_capacity=int(n / 0.9), window_width=W)
+        api.wc_insert(t.handle, keys[:n], keys[:n])
+        q = keys[n // 2:n + n // 2].contiguous()
+        out, found = torch.empty_like(q), torch.empty(n, dtype=torch.uint8, device="cuda")
+        us.append(_graph_us(lambda: api.wc_retrieve(t.handle, q, out, found), 20))
+        assert bool(found[:n - n // 2].all())
+    assert us[1] < 2 * us[0], us
