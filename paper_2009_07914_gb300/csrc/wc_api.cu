@@ -250,7 +250,10 @@ bool stream_capturing(cudaStream_t s) {
 }
 
 cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, uint64_t likely) {
-  if (t->scratch_ev != nullptr && t->scratch_stream != s && !stream_capturing(s)) {
+  // also on the stream of the last call: two streams can share a handle (the per-thread default
+  // stream of two threads; one destroyed with work pending and one created after it), and a
+  // wait that is already met costs nothing on the device
+  if (t->scratch_ev != nullptr && !stream_capturing(s)) {
     const cudaError_t e = cudaStreamWaitEvent(s, t->scratch_ev, 0);
     if (e != cudaSuccess) return e;
   }
@@ -283,7 +286,6 @@ cudaError_t scratch_release(const wc_table* t, cudaStream_t s) {
     const cudaError_t e = cudaEventCreateWithFlags(&t->scratch_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
   }
-  t->scratch_stream = s;
   return cudaEventRecord(t->scratch_ev, s);
 }
 

@@ -146,7 +146,6 @@ struct wc_table {
   mutable void* d_scratch;
   mutable uint64_t scratch_bytes;
   mutable cudaEvent_t scratch_ev = nullptr;  // end of the last call that used the scratch
-  mutable cudaStream_t scratch_stream = nullptr;  // and its stream
   wc::HostPipe* host = nullptr;  // host-buffer pipeline, created on first use
 };
 
