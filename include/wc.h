@@ -219,7 +219,9 @@ typedef struct {
  * active part of the table stays in L2; needs scratch of n * (key + value) bytes (lookups:
  * n * (key + value + 3) bytes and 8 bytes per 4096 queries and region), which the table
  * allocates on first use (stream-ordered) and keeps; calls that share it on different
- * streams are ordered one behind the other.  Inserts of single-value,
+ * streams are ordered one behind the other.  Calls recorded into CUDA graphs (these inserts,
+ * and every insert of counting and bucket multi-value tables) share a second buffer of the
+ * table, kept until it is destroyed; the caller orders the replays that use it.  Inserts of single-value,
  * counting, hash-set and open-addressing multi-value tables; retrieves of single-value and
  * counting tables (the results are put back in input order).  WC_SCHEME_AUTO picks
  * BLOCKED for those inserts when the batch holds at least 2^18 pairs and the table is

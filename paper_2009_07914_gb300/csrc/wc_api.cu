@@ -249,14 +249,55 @@ bool stream_capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
-cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, uint64_t likely) {
+// Scratch of a call that is being recorded into a CUDA graph.  The graph keeps the address, so
+// the buffer is one that only recorded calls use and that lives as long as the table: the
+// buffer that a warm-up call left behind is taken over once its last call is done (recording
+// then allocates nothing), else one is allocated now, outside the graph.  A buffer that is
+// too small stays for the graphs that hold it.
+static cudaError_t recorded_scratch(const wc_table* t, uint64_t bytes, char** out) {
+  if (bytes <= t->recorded_bytes) {
+    *out = static_cast<char*>(t->recorded.back());
+    return cudaSuccess;
+  }
+  // the capture forbids this thread neither the wait nor the allocation
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  void* p = nullptr;
+  uint64_t got = 0;
+  if (bytes <= t->scratch_bytes) {
+    if (t->scratch_ev != nullptr) e = cudaEventSynchronize(t->scratch_ev);
+    if (e == cudaSuccess) {
+      p = t->d_scratch;
+      got = t->scratch_bytes;
+      t->d_scratch = nullptr;
+      t->scratch_bytes = 0;
+    }
+  } else if (injected_alloc_failure()) {
+    e = cudaErrorMemoryAllocation;
+  } else {
+    got = align_up(bytes, kAlign);
+    e = cudaMalloc(&p, got);
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);  // back
+  if (e != cudaSuccess) return e;
+  t->recorded.push_back(p);
+  t->recorded_bytes = got;
+  t->recorded_total += got;
+  *out = static_cast<char*>(p);
+  return cudaSuccess;
+}
+
+cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, char** out, uint64_t likely) {
+  if (stream_capturing(s)) return recorded_scratch(t, bytes, out);
   // also on the stream of the last call: two streams can share a handle (the per-thread default
   // stream of two threads; one destroyed with work pending and one created after it), and a
   // wait that is already met costs nothing on the device
-  if (t->scratch_ev != nullptr && !stream_capturing(s)) {
+  if (t->scratch_ev != nullptr) {
     const cudaError_t e = cudaStreamWaitEvent(s, t->scratch_ev, 0);
     if (e != cudaSuccess) return e;
   }
+  *out = static_cast<char*>(t->d_scratch);
   if (bytes <= t->scratch_bytes) return cudaSuccess;
   if (t->d_scratch != nullptr) {
     cudaError_t e = cudaFreeAsync(t->d_scratch, s);
@@ -277,6 +318,7 @@ cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, ui
     return e;
   }
   t->scratch_bytes = want;
+  *out = static_cast<char*>(t->d_scratch);
   return cudaSuccess;
 }
 
@@ -605,9 +647,10 @@ wc_status wc_table_destroy(wc_table* t) {
   DeviceGuard guard(t->device);
   host_pipe_free(t);
   l2_carveout_release(t);
-  if (t->d_scratch != nullptr) {
+  if (t->d_scratch != nullptr || !t->recorded.empty()) {
     cudaDeviceSynchronize();
     cudaFree(t->d_scratch);
+    for (void* p : t->recorded) cudaFree(p);
   }
   if (t->scratch_ev != nullptr) cudaEventDestroy(t->scratch_ev);
   cudaError_t e = cudaFree(t->d_block);
@@ -634,7 +677,7 @@ wc_status wc_table_get_info(const wc_table* t, wc_table_info* h_out) {
   h_out->kind = t->cfg.kind;
   h_out->options = t->cfg.options;
   h_out->reserved = 0;
-  h_out->work_bytes = t->scratch_bytes + host_pipe_bytes(t);
+  h_out->work_bytes = t->scratch_bytes + t->recorded_total + host_pipe_bytes(t);
   return WC_OK;
 }
 

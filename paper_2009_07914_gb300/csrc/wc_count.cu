@@ -133,9 +133,10 @@ cudaError_t aggregate(const wc_table* t, const void* keys, const void* weights, 
                       bool dense, const void** akeys, const void** avals, const unsigned long long** n_dev,
                       cudaStream_t s) {
   const uint64_t kbytes = (n * sizeof(K) + 255) / 256 * 256;
-  cudaError_t e = ensure_scratch(t, skip_bytes + 256 + kbytes + n * sizeof(V), s);
+  char* sc = nullptr;
+  cudaError_t e = ensure_scratch(t, skip_bytes + 256 + kbytes + n * sizeof(V), s, &sc);
   if (e != cudaSuccess) return e;
-  auto* cursor = reinterpret_cast<unsigned long long*>(static_cast<char*>(t->d_scratch) + skip_bytes);
+  auto* cursor = reinterpret_cast<unsigned long long*>(sc + skip_bytes);
   K* ok = reinterpret_cast<K*>(reinterpret_cast<char*>(cursor) + 256);
   V* ov = reinterpret_cast<V*>(reinterpret_cast<char*>(ok) + kbytes);
   if (dense) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "wc.h"
 
@@ -146,6 +147,9 @@ struct wc_table {
   mutable void* d_scratch;
   mutable uint64_t scratch_bytes;
   mutable cudaEvent_t scratch_ev = nullptr;  // end of the last call that used the scratch
+  mutable std::vector<void*> recorded;  // scratch of calls recorded into graphs, the last one in use
+  mutable uint64_t recorded_bytes = 0;  // bytes of the last one
+  mutable uint64_t recorded_total = 0;  // and of all
   wc::HostPipe* host = nullptr;  // host-buffer pipeline, created on first use
 };
 
@@ -176,12 +180,14 @@ uint64_t scan_partials_needed(uint64_t n);
 
 int sm_count_of(int device);
 
-// Scratch of at least `bytes` on stream s (grows the table's buffer if needed), ordered
-// behind the last call that used it: calls of the same kind may overlap on different
+// Scratch of at least `bytes` on stream s, in *out (grows the table's buffer if needed),
+// ordered behind the last call that used it: calls of the same kind may overlap on different
 // streams, and there is one buffer per table.  scratch_release marks the end of this call's
-// use of it (after its last kernel).  Inside a stream capture neither touches the event.
+// use of it (after its last kernel).  Inside a stream capture neither touches the event: the
+// calls recorded into graphs share a buffer of their own, which no other call uses and which
+// is kept until the table is destroyed.
 // likely: bytes that calls expected next will need, taken along when the buffer grows.
-cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, uint64_t likely = 0);
+cudaError_t ensure_scratch(const wc_table* t, uint64_t bytes, cudaStream_t s, char** out, uint64_t likely = 0);
 cudaError_t scratch_release(const wc_table* t, cudaStream_t s);
 
 // Whether s is being captured into a graph.

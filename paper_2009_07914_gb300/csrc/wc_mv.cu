@@ -54,9 +54,8 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
     counters = sp.counters;
     rec_base = sp.extra;
   } else {
-    e = ensure_scratch(t, rec_bytes, s);
+    e = ensure_scratch(t, rec_bytes, s, &rec_base);
     if (e != cudaSuccess) return e;
-    rec_base = static_cast<char*>(t->d_scratch);
   }
   TileRecord rec;
   rec.list = reinterpret_cast<uint2*>(rec_base);

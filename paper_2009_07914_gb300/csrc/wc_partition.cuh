@@ -399,9 +399,9 @@ cudaError_t region_split(const wc_table* t, const RegionMap& m, const K* keys, c
   const uint64_t keys_off = kSplitHeader;
   const uint64_t vals_off = keys_off + align256(n * sizeof(K));
   const uint64_t extra_off = vals_off + (kVals == kValsNone ? 0 : align256(n * sizeof(V)));
-  cudaError_t e = ensure_scratch(t, extra_off + extra, s, lookup_scratch_likely(t, n));
+  char* sc = nullptr;
+  cudaError_t e = ensure_scratch(t, extra_off + extra, s, &sc, lookup_scratch_likely(t, n));
   if (e != cudaSuccess) return e;
-  char* sc = static_cast<char*>(t->d_scratch);
   out.keys = reinterpret_cast<K*>(sc + keys_off);
   out.vals = kVals == kValsNone ? nullptr : reinterpret_cast<V*>(sc + vals_off);
   auto* hist = reinterpret_cast<unsigned int*>(sc + kSplitHist);
