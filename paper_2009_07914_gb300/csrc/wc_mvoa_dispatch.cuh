@@ -17,7 +17,9 @@ cudaError_t oa_run(const wc_table* t, int op, const void* keys, const void* vals
   const wc_launch& lc = t->launch[op];
   const int block = lc.block_threads;
   TableDesc d = desc_of(t);
-  d.ovf = t->walk_off ? nullptr : t->d_walk;
+  // A count recorded into a graph does not use the walk bits: between its replays the slots may
+  // be handed to a user kernel, which sets none (recorded inserts do set them).
+  d.ovf = t->walk_off || (op == WC_OP_COUNT && stream_capturing(s)) ? nullptr : t->d_walk;
   const Key* k = static_cast<const Key*>(keys);
   constexpr int W = G * S;
   if (op == WC_OP_INSERT) {

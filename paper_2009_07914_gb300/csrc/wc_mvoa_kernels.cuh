@@ -20,7 +20,8 @@
 // there, so a counting walk may stop at a full window whose bit for its tag is clear (it went
 // on to a window with an empty slot, and a random window is a line from HBM: 2^26 pairs, four
 // per key, load 0.8, 2^26 queries, three quarters of them absent, 3.93 -> 2.43 ms).  In a
-// table whose slots a user's kernel may have written t.ovf is null, and walks go on.
+// table whose slots a user's kernel may have written t.ovf is null, and walks go on; so they do
+// in counts recorded into a graph.
 #pragma once
 
 #include "wc_device.cuh"

@@ -91,3 +91,56 @@ def test_counts_split_by_region(wc, bucket):
         assert torch.equal(a[i:i + part.numel() + 1], b[:part.numel() + 1] + at)
         at += s
     assert total == at == int(a[m])
+
+
+M64 = (1 << 64) - 1
+
+
+def _first_two_windows(key, seed, p):
+    k = (key ^ seed) & M64
+    k ^= k >> 33
+    k = (k * 0xFF51AFD7ED558CCD) & M64
+    k ^= k >> 33
+    k = (k * 0xC4CEB9FE1A85EC53) & M64
+    k ^= k >> 33
+    w = ((k >> 32) * p) >> 32
+    return w, (w + 1 + (((k & 0xFFFFFFFF) * (p - 1)) >> 32)) % p
+
+
+@pytest.mark.parametrize("W", [8, 16])
+def test_recorded_count_sees_slots_that_a_user_kernel_wrote(wc, W):
+    """A count is recorded, then the table's slots are handed out and a pair is put into the
+    second window of its key without a walk bit (as a user kernel would; written here by a
+    copy): the replay and a new count both find it."""
+    import ctypes
+
+    import torch
+    from paper_2009_07914_gb300 import api
+    seed = 0x5EED_C0DE
+    t = wc.MultiValueOATable(4, 4, min_capacity=11 * W, window_width=W, seed=seed)
+    p = t.info["windows"]
+    by_first = {}
+    for k in range(1, 5000):
+        by_first.setdefault(_first_two_windows(k, seed, p)[0], []).append(k)
+    w0, group = max(by_first.items(), key=lambda x: len(x[1]))
+    fill, key = group[:W], next(k for k in group[W:] if _first_two_windows(k, seed, p)[1] != w0)
+    t.insert(np.array(fill, np.uint32), np.zeros(W, np.uint32))  # the window is full, none walked past it
+    q = torch.tensor([key, fill[0]], dtype=torch.int32, device="cuda")
+    offs = torch.empty(3, dtype=torch.int64, device="cuda")
+    assert api.wc_count_values(t.handle, q, offs) == 1  # the kernels are loaded before the capture
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        api.wc_count_values(t.handle, q, offs, want_total=False)
+    g.replay()
+    assert offs.tolist() == [0, 0, 1]
+    view = api.wc_table_device_view(t.handle)
+    word = torch.tensor([5 << 32 | key], dtype=torch.int64, device="cuda")
+    slot = view.slots + 8 * W * _first_two_windows(key, seed, p)[1]
+    torch.cuda.synchronize()
+    rt = ctypes.CDLL("libcudart.so.13")  # the runtime instance libwc.so is linked against
+    assert rt.cudaMemcpy(ctypes.c_void_p(slot), ctypes.c_void_p(word.data_ptr()), ctypes.c_size_t(8), 3) == 0
+    offs.fill_(-1)
+    g.replay()
+    assert offs.tolist() == [0, 1, 2]
+    assert api.wc_count_values(t.handle, q, offs) == 2 and offs.tolist() == [0, 1, 2]
