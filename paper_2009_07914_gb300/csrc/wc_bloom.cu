@@ -233,8 +233,7 @@ cudaError_t insert(const wc_table* t, const K* keys, uint64_t n, cudaStream_t s)
       if (fill) {
         auto kern = k_bloom_fill<K>;
         const size_t smem = (32ull << m.shift) + fill_words(m.R) * 4;
-        static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                             (32 << 12) + fill_words(kMaxSplitRegions) * 4);
+        const cudaError_t attr = allow_smem(kern, (32 << 12) + fill_words(kMaxSplitRegions) * 4);
         const uint64_t part = std::min(std::max<uint64_t>(4 * (n / m.R + 1), 4ull << m.shift), kFillPart);
         const unsigned grid = static_cast<unsigned>(occupancy_smem(kern, kFillThreads, smem) * t->sm_count);
         e = attr != cudaSuccess ? attr

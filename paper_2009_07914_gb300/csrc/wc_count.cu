@@ -142,11 +142,8 @@ cudaError_t aggregate(const wc_table* t, const void* keys, const void* weights, 
   if (dense) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   auto kern = k_count_aggregate<K, V>;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(count_agg_smem<K, V>()));
-    attr = true;
-  }
+  e = allow_smem(kern, count_agg_smem<K, V>());
+  if (e != cudaSuccess) return e;
   const uint64_t ntiles = (n + kCntTile - 1) / kCntTile;
   const uint64_t most = static_cast<uint64_t>(occupancy_smem(kern, kCntThreads, count_agg_smem<K, V>())) * t->sm_count;
   kern<<<static_cast<unsigned>(ntiles < most ? ntiles : most), kCntThreads, count_agg_smem<K, V>(), s>>>(

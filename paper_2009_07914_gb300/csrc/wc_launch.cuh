@@ -24,6 +24,16 @@ int occupancy_smem(Kernel kernel, int block, size_t smem) {
   return occupancy_cached(reinterpret_cast<const void*>(kernel), block, smem);
 }
 
+// Lets the kernel take up to `bytes` of dynamic shared memory on the current device.  Set on
+// every call: the limit belongs to the device's context, so one set once per process is
+// missing on a second device and after cudaDeviceReset (0.2 us a call).  `bytes` is the
+// kernel's constant maximum, not the launch's own need: another thread may be between its call
+// of this and its launch.
+template <class F>
+cudaError_t allow_smem(F kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+}
+
 // Persistent-style grid for the probe engines: at most blocks_per_sm * SMs blocks, and
 // no more warps than one key per group needs; each warp owns `per_warp` consecutive
 // input positions.

@@ -19,11 +19,8 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
   auto count = k_mv_aggregate<KIn, W, kThreads>;
   auto place = k_mv_place<VB, kThreads>;
   const size_t smem_c = A::smem_bytes(sizeof(KIn));
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaFuncSetAttribute(count, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_c));
-    attr_done = true;
-  }
+  cudaError_t e = allow_smem(count, smem_c);
+  if (e != cudaSuccess) return e;
   // The counting pass's record for the placing pass (TileRecord): a (slot, count) entry
   // per distinct key of a tile and one word per element.
   const uint64_t ntiles = (n + A::kTile - 1) / A::kTile;
@@ -38,7 +35,6 @@ cudaError_t insert_passes(const wc_table* t, const void* keys, const void* vals,
   // (pass 2 lays buckets out in key-store order).
   unsigned long long* counters = nullptr;
   char* rec_base = nullptr;
-  cudaError_t e = cudaSuccess;
   if (n >= (1ull << 20) && t->table_bytes > (64ull << 20)) {
     RegionSplit<KIn, V> sp;
     // About 128 regions rather than L2-sized ones: a tile of one region then holds fewer

@@ -371,12 +371,8 @@ cudaError_t split_launch(const wc_table* t, const RegionMap& m, const K* keys, c
   const uint32_t copies = hist_copies(m.R);
   const size_t hsm = static_cast<size_t>(copies) * m.R * sizeof(unsigned int);
   const size_t ssm = Tile::smem_bytes(m.R, kTile);
-  static const cudaError_t attr = [&] {
-    const cudaError_t e = cudaFuncSetAttribute(hk, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistWarps * 512 * 4);
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(Tile::smem_bytes(kMaxSplitRegions, kTile)));
-  }();
+  static_assert(kHistWarps * 512 * 4 <= 48 << 10, "the histogram needs no raised limit");
+  const cudaError_t attr = allow_smem(sk, Tile::smem_bytes(kMaxSplitRegions, kTile));
   if (attr != cudaSuccess) return attr;
   const uint64_t hist_most = static_cast<uint64_t>(occupancy_smem(hk, kPartThreads, hsm)) * t->sm_count;
   const uint64_t split_most = static_cast<uint64_t>(occupancy_smem(sk, kPartThreads, ssm)) * t->sm_count;
