@@ -116,7 +116,7 @@ template <class K>
 __global__ void __launch_bounds__(kFillThreads) k_bloom_fill(TableDesc t, const K* __restrict__ keys, RegionMap m,
                                                              const unsigned int* __restrict__ hist, uint32_t part,
                                                              unsigned long long* next_unit, int k) {
-  extern __shared__ unsigned long long fill_smem[];
+  extern __shared__ __align__(16) unsigned long long fill_smem[];
   const uint32_t words = 4u << m.shift;  // 64-bit words of a region
   unsigned long long* s_bits = fill_smem;
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(fill_smem + words);

@@ -49,7 +49,7 @@ template <class K, class V>
 __global__ void __launch_bounds__(kCntThreads) k_count_aggregate(const K* __restrict__ keys, const V* __restrict__ w,
                                                                  uint64_t n, K* __restrict__ ok, V* __restrict__ ov,
                                                                  uint32_t* status, unsigned long long* cursor) {
-  extern __shared__ unsigned long long cnt_smem[];
+  extern __shared__ __align__(16) unsigned long long cnt_smem[];
   K* s_key = reinterpret_cast<K*>(cnt_smem);
   V* s_sum = reinterpret_cast<V*>(s_key + kCntSlots);
   __shared__ uint32_t s_warp[kCntThreads / 32];

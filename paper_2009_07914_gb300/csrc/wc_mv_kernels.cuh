@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
                                                               TileRecord rec) {
   constexpr int kAggTile = Agg<kAggThreads>::kTile;
   constexpr int kAggSlots = Agg<kAggThreads>::kSlots;
-  extern __shared__ unsigned long long agg_smem[];  // Agg<kAggThreads>::smem_bytes(sizeof(KIn)) bytes
+  extern __shared__ __align__(16) unsigned long long agg_smem[];  // Agg<kAggThreads>::smem_bytes(sizeof(KIn)) bytes
   unsigned long long* s_key = agg_smem;
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(agg_smem + kAggSlots);
   uint32_t* s_ks = s_cnt + kAggSlots;  // key-store slot of every list entry (kAggTile)

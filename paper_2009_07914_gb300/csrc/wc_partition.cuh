@@ -64,7 +64,7 @@ template <class K>
 __global__ void __launch_bounds__(kPartThreads) k_part_hist(const K* __restrict__ keys, uint64_t n, RegionMap m,
                                                             unsigned int* __restrict__ hist, uint32_t copies,
                                                             const unsigned long long* n_dev) {
-  extern __shared__ unsigned int s_hw[];  // copies * R
+  extern __shared__ __align__(16) unsigned int s_hw[];  // copies * R
   if (n_dev != nullptr) n = *n_dev;
   for (uint32_t i = threadIdx.x; i < copies * m.R; i += kPartThreads) s_hw[i] = 0;
   __syncthreads();
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kPartThreads, (SplitTile<K, V, kVals>::kMinBlo
   using Tile = SplitTile<K, V, kVals>;
   constexpr bool kPreKey = Tile::kPreKey, kPreVal = Tile::kPreVal, kPre = kPreKey || kPreVal, kRead = Tile::kRead;
   constexpr int kTile = kPartThreads * kItems;
-  extern __shared__ unsigned long long scatter_smem[];
+  extern __shared__ __align__(16) unsigned long long scatter_smem[];
   char* at = reinterpret_cast<char*>(scatter_smem);
   auto carve = [&](size_t bytes) {
     char* p = at;
