@@ -179,8 +179,12 @@ template <int kSlots>
 __device__ __forceinline__ int smem_find_or_insert(unsigned long long* s_key, unsigned long long key, bool& fresh) {
   volatile unsigned long long* vk = s_key;
   // Fibonacci hashing: the table lives for one tile, and the keys of a tile come from
-  // everywhere (a full mix cost more than the few collisions it saves)
-  uint32_t h = static_cast<uint32_t>((key * 0x9E3779B97F4A7C15ull) >> 40) & (kSlots - 1);
+  // everywhere (a full mix cost more than the few collisions it saves).  The top bits of the
+  // product, which depend on every bit of the key: lower ones are the same for keys that
+  // differ only above them (1024 keys i << 52 would be one chain).
+  constexpr int kShift = 64 - (kSlots == 2048 ? 11 : 12);
+  static_assert(kSlots == 2048 || kSlots == 4096, "slots of a tile's table");
+  uint32_t h = static_cast<uint32_t>((key * 0x9E3779B97F4A7C15ull) >> kShift);
   while (true) {  // at most kSlots / 2 distinct keys in a table of kSlots slots
     const unsigned long long cur = vk[h];
     if (cur == key) return static_cast<int>(h);
