@@ -169,7 +169,13 @@ struct LayoutP32 {
   __device__ static Slot tomb() { return Slot{0xffffffffull}; }
   __device__ static Slot from_words(const unsigned long long* u) { return Slot{u[0]}; }
   __device__ static bool cas(Slot* p, const Slot& e, const Slot& d) {
-    return atomicCAS(&p->w, e.w, d.w) == e.w;
+    Slot seen;
+    return cas(p, e, d, seen);
+  }
+  // the same, leaving in `seen` the word that it found
+  __device__ static bool cas(Slot* p, const Slot& e, const Slot& d, Slot& seen) {
+    seen.w = atomicCAS(&p->w, e.w, d.w);
+    return seen.w == e.w;
   }
   __device__ static void store_val(Slot* p, Val v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(reinterpret_cast<uint32_t*>(&p->w) + 1), "r"(v)
@@ -202,17 +208,20 @@ struct LayoutP64 {
   __device__ static Slot tomb() { return Slot{~0ull, 0ull}; }
   __device__ static Slot from_words(const unsigned long long* u) { return Slot{u[0], u[1]}; }
   __device__ static bool cas(Slot* p, const Slot& e, const Slot& d) {
-    unsigned long long olo, ohi;
+    Slot seen;
+    return cas(p, e, d, seen);
+  }
+  __device__ static bool cas(Slot* p, const Slot& e, const Slot& d, Slot& seen) {
     asm volatile(
         "{\n\t.reg .b128 e, d, o;\n\t"
         "mov.b128 e, {%2, %3};\n\t"
         "mov.b128 d, {%4, %5};\n\t"
         "atom.global.cas.b128 o, [%6], e, d;\n\t"
         "mov.b128 {%0, %1}, o;\n\t}"
-        : "=l"(olo), "=l"(ohi)
+        : "=l"(seen.k), "=l"(seen.v)
         : "l"(e.k), "l"(e.v), "l"(d.k), "l"(d.v), "l"(p)
         : "memory");
-    return olo == e.k && ohi == e.v;
+    return seen.k == e.k && seen.v == e.v;
   }
   __device__ static void store_val(Slot* p, Val v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&p->v), "l"(v) : "memory");
@@ -255,6 +264,10 @@ struct LayoutK64 {
   __device__ static Slot tomb() { return Slot{~0ull}; }
   __device__ static Slot from_words(const unsigned long long* u) { return Slot{u[0]}; }
   __device__ static bool cas(Slot* p, const Slot& e, const Slot& d) { return atomicCAS(&p->k, e.k, d.k) == e.k; }
+  __device__ static bool cas(Slot* p, const Slot& e, const Slot& d, Slot& seen) {
+    seen.k = atomicCAS(&p->k, e.k, d.k);
+    return seen.k == e.k;
+  }
   __device__ static void store_val(Slot*, Val) {}
   __device__ static Slot shfl(const Slot& s, int src) { return Slot{__shfl_sync(kFull, s.k, src)}; }
 };
@@ -276,6 +289,10 @@ struct LayoutK32 {
   __device__ static Slot make(Key k, Val) { return Slot{k}; }
   __device__ static Slot tomb() { return Slot{0xffffffffu}; }
   __device__ static bool cas(Slot* p, const Slot& e, const Slot& d) { return atomicCAS(&p->k, e.k, d.k) == e.k; }
+  __device__ static bool cas(Slot* p, const Slot& e, const Slot& d, Slot& seen) {
+    seen.k = atomicCAS(&p->k, e.k, d.k);
+    return seen.k == e.k;
+  }
   __device__ static void store_val(Slot*, Val) {}
   __device__ static Slot shfl(const Slot& s, int src) { return Slot{__shfl_sync(kFull, s.k, src)}; }
 };

@@ -4,17 +4,24 @@
 // Swept region by region (or into a table that fits L2) an insert is bound by the L2's rate
 // of window reads followed by CASes (ldcg1 ff. in wc_device.cuh: 68 G/s at best) and by its
 // chain of those two round trips.  The first window of a key takes most of them, so it is
-// probed straight from the input; pairs that are not placed there (a full window, a lost
-// race for a slot) go to the warp's queue in shared memory and are worked on 32 at a time.
-// The claim rules are those of sv_insert_range (the group-per-key engine that wider windows
-// run on): the earliest candidate of the key's sequence once the walk has met an empty slot
-// or its end.
+// probed straight from the input; pairs that are not placed there (a full window, a slot lost
+// to another pair and no other in the window) go to the warp's queue in shared memory and are
+// worked on 32 at a time.  The claim rules are those of sv_insert_range (the group-per-key
+// engine that wider windows run on): the earliest candidate of the key's sequence once the
+// walk has met an empty slot or its end.
 //
 // The sweep of 2^27 pairs, one GB300, that engine against this kernel (with half-line
 // reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.86 ms (2.63 with the table
-// copied to L2 ahead of the sweep, BatchBlocks::prefetch), at 0.5 3.11 -> 2.30; 8+8 bytes at 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.  In input order, 2^20
-// pairs at 0.9 65.7 -> 65.6 us, at 0.5 44.0 -> 40.1; half a table erased and inserted again
-// (2^20 keys, 0.9) 172 -> 118 us.
+// copied to L2 ahead of the sweep, BatchBlocks::prefetch), at 0.5 3.11 -> 2.30; 8+8 bytes at
+// 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.
+//
+// In input order it is races for slots that take the time: all pairs of a batch into a fresh
+// table want the first slots of its windows at once.  A pair that loses one tries the next of
+// the window with another CAS and nothing read in between; reading window and slot again for
+// each lost race was slower than the group engine.  131,072 pairs of 4+4 bytes, load 0.6, that
+// engine / read again / next slot 18.8 / 21.6 / 14.6 us, at 0.9 32.4 / 35.4 / 27.4; 2^20 at
+// 0.9 55.9 / 53.3 / 52.0; 1000 at 0.6 14.8 / 15.2 / 8.6; sets of 8-byte keys, 222,476 at 0.9
+// 34.7 / 39.7 / 33.2.
 #pragma once
 
 #include "wc_launch.cuh"
@@ -27,23 +34,24 @@ namespace wc {
 struct Spot {
   uint32_t at;    // slot of the key (hit)
   uint32_t tomb;  // first tombstone (has_tomb)
-  uint32_t used;  // slots that are not empty: the empty ones are the last ones (probe_window)
+  uint32_t empty;  // first empty slot, W when there is none
   bool hit, has_tomb;
 };
 
 // S slots, the first of them slot `first` of the window, in one word: bit 0 the key is here,
-// bit 1 a tombstone is, bits 2..7 the key's slot, 8..13 the first tombstone, 14.. slots in use.
+// bit 1 a tombstone is, bits 2..7 the key's slot, 8..13 the first tombstone, 14.. the first
+// empty slot, first + S when there is none.
 template <class L, int S>
 __device__ __forceinline__ uint32_t spot_word(const typename L::Slot (&s)[S], typename L::Key k, uint32_t first) {
-  uint32_t hit = 0, tomb = 0, used = 0;
+  uint32_t hit = 0, tomb = 0, empty = (first + S) << 14;
 #pragma unroll
   for (int i = S - 1; i >= 0; --i) {
     const typename L::Key kk = L::key(s[i]);
     if (kk == k) hit = 1u | (first + i) << 2;
     if (kk == L::kTomb) tomb = 2u | (first + i) << 8;
-    if (kk != L::kEmpty) used += 1u << 14;
+    if (kk == L::kEmpty) empty = (first + i) << 14;
   }
-  return hit | tomb | used;
+  return hit | tomb | empty;
 }
 
 // Window w seen by the key k; every lane of the warp calls, with a window of the table.  As in
@@ -51,7 +59,7 @@ __device__ __forceinline__ uint32_t spot_word(const typename L::Slot (&s)[S], ty
 template <class L, int W>
 __device__ __forceinline__ Spot spot_of(const typename L::Slot* slots, typename L::Key k, uint32_t w) {
   using Slot = typename L::Slot;
-  uint32_t lo, hi = 0;  // the window's first half (or all of it), its second
+  uint32_t lo, hi = W << 14;  // the window's first half (or all of it), its second
   if constexpr (W * slot_size<L>() <= 32) {
     Slot s[W];
     load_slots<L, W, true>(slots + static_cast<uint64_t>(w) * W, s);
@@ -75,20 +83,9 @@ __device__ __forceinline__ Spot spot_of(const typename L::Slot* slots, typename 
   r.has_tomb = (lo | hi) & 2u;
   r.at = ((lo | hi) >> 2) & 63u;  // the key is in one half at most
   r.tomb = ((lo & 2u ? lo : hi) >> 8) & 63u;
-  r.used = (lo >> 14) + (hi >> 14);
+  r.empty = lo >> 14;
+  if (W * slot_size<L>() > 32 && r.empty == W / 2) r.empty = hi >> 14;
   return r;
-}
-
-// One slot, bypassing L1.
-template <class L>
-__device__ __forceinline__ typename L::Slot slot_now(const typename L::Slot* p) {
-  if constexpr (L::kHalf) {
-    return typename L::Slot{__ldcg(reinterpret_cast<const uint32_t*>(p))};
-  } else {
-    typename L::Slot s[1];
-    load_slots<L, 1, true>(p, s);
-    return s[0];
-  }
 }
 
 template <class Key, class Val>
@@ -109,9 +106,8 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
   using Slot = typename L::Slot;
   using Key = typename L::Key;
   using Val = typename L::Val;
-  // first tombstone of a walk: none; none, and the pair has lost a slot before; its index,
-  // with kReread when the pair has lost a slot before
-  constexpr uint64_t kNone = ~0ull, kLost = ~1ull, kReread = 1ull << 62;
+  // first tombstone of a walk: none; none, and the pair has lost a slot before; else its index
+  constexpr uint64_t kNone = ~0ull, kLost = ~1ull;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   Slot* slots = static_cast<Slot*>(t.slots);
@@ -125,52 +121,67 @@ __device__ __forceinline__ void insert_blocks(const TableDesc& t, const typename
     uint32_t w, j;
     uint64_t tomb, h;
   };
-  // One window of the walk, in every lane with `on` (cleared when the pair is done).  A free
-  // slot is taken to hold the word that clears and erases leave; a pair that has lost a slot
-  // reads the word again before its CAS.
+  // One window of the walk, in every lane with `on` (cleared when the pair is done).
   auto step = [&](bool& on, Pair& x) {
     const Spot s = spot_of<L, W>(slots, x.k, x.w);
     if (!on) return;
     const uint64_t base = static_cast<uint64_t>(x.w) * W;
-    if (s.hit) {  // overwrite the value (duplicate warning, Sec. IV-B3)
-      slot_store_value<L>(slots, t.vals, base + s.at, x.v);
+    auto stored = [&](uint64_t at) {  // the key is there: overwrite the value (duplicate warning, Sec. IV-B3)
+      slot_store_value<L>(slots, t.vals, at, x.v);
       if constexpr (!L::kCount) flags |= kFlagDuplicate;
       on = false;
+    };
+    if (s.hit) {
+      stored(base + s.at);
       return;
     }
     // A pair that lost a slot has walked to its end without meeting the key, so the first
     // free slot it meets now is its own: had a copy of the key gone to a later window since,
     // it would have passed that free slot (tombstones only get fewer during an insert).
     const bool at_once = x.tomb == kLost && s.has_tomb;
-    if (s.has_tomb && x.tomb >= kLost) x.tomb = (base + s.tomb) | (x.tomb == kLost ? kReread : 0ull);
+    if (s.has_tomb && x.tomb >= kLost) x.tomb = base + s.tomb;
     const bool from_tomb = x.tomb < kLost;
-    if (s.used == W && x.j + 1 < t.p && !at_once) {  // no empty slot: walk on
+    if (s.empty == W && x.j + 1 < t.p && !at_once) {  // no empty slot: walk on
       if (t.ovf != nullptr) ovf_mark(t.ovf, x.w, static_cast<uint32_t>(x.h) & 7u);
       x.w = probe_next(x.w, 1u + __umulhi(static_cast<uint32_t>(x.h), t.p - 1u), t.p);
       ++x.j;
       return;
     }
-    if (!from_tomb && s.used == W) {
+    if (!from_tomb && s.empty == W) {
       flags |= kFlagProbeLimit;  // every window visited, nothing to claim
       on = false;
       return;
     }
-    // claim the earliest candidate: the remembered tombstone, else the first empty slot
-    const uint64_t c = from_tomb ? x.tomb & ~kReread : base + s.used;
+    // Claim the earliest candidate: the remembered tombstone, else the first empty slot, taken
+    // to hold the word that clears and erases leave.  Where the slot went to another key, the
+    // next one of the window is tried at once: slots fill in order, so the key is in none
+    // behind the one that is claimed, and every one before it was seen here or by a CAS.
+    uint64_t c = from_tomb ? x.tomb : base + s.empty;
+    const uint64_t last = from_tomb ? c : base + (W - 1);
     Slot old = from_tomb ? L::tomb() : Slot{};
-    bool ok = true;
-    if (from_tomb ? (x.tomb & kReread) != 0 : x.tomb == kLost) {
-      old = slot_now<L>(slots + c);
-      ok = L::key(old) == (from_tomb ? L::kTomb : L::kEmpty);
+    const Slot pair = L::make(x.k, x.v);
+    while (true) {
+      Slot seen;
+      if (L::cas(slots + c, old, pair, seen)) {
+        if constexpr (L::kSoA) slot_store_value<L>(slots, t.vals, c, x.v);
+        ++added;
+        on = false;
+        return;
+      }
+      const Key kk = L::key(seen);
+      if (kk == x.k) {  // by another copy of the pair's key
+        stored(c);
+        return;
+      }
+      if (kk == (from_tomb ? L::kTomb : L::kEmpty)) {
+        old = seen;  // still free, with another word
+        continue;
+      }
+      if (c == last) break;
+      ++c;
+      old = Slot{};
     }
-    if (ok) ok = L::cas(slots + c, old, L::make(x.k, x.v));
-    if (ok) {
-      if constexpr (L::kSoA) slot_store_value<L>(slots, t.vals, c, x.v);
-      ++added;
-      on = false;
-      return;
-    }
-    // another pair took it: on from the slot's window (the ones before it hold no free slot)
+    // on from the slot's window (the ones before it hold no free slot)
     x.w = static_cast<uint32_t>(c / W);
     if (from_tomb) x.j = 0;
     x.tomb = kLost;

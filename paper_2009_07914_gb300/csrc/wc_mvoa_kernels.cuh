@@ -292,6 +292,18 @@ __device__ __forceinline__ uint32_t oa_window(const typename L::Slot* slots, typ
   }
 }
 
+// One slot, bypassing L1.
+template <class L>
+__device__ __forceinline__ typename L::Slot slot_now(const typename L::Slot* p) {
+  if constexpr (L::kHalf) {
+    return typename L::Slot{__ldcg(reinterpret_cast<const uint32_t*>(p))};
+  } else {
+    typename L::Slot s[1];
+    load_slots<L, 1, true>(p, s);
+    return s[0];
+  }
+}
+
 // A batch split by table region, swept in order.  2^26 pairs, four per key, load 0.8: the
 // sweep 2.02 -> 1.81 ms (k_oa_insert, 2.17 with the walk bits).
 template <class L, int W>

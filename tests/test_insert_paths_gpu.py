@@ -114,3 +114,59 @@ def test_sweeps_of_every_chunk_length(wc, kb, n, load):
     out, found, _ = t.retrieve(keys)
     assert found.all()
     np.testing.assert_array_equal(out, vals)
+
+
+@pytest.mark.parametrize("kb,W", [(4, 8), (4, 4), (8, 4), (8, 2)])
+@pytest.mark.parametrize("windows,copies", [(7, 1), (7, 40), (1009, 8), (40_009, 3)])
+def test_pairs_that_race_for_the_same_slots(wc, kb, W, windows, copies):
+    """Every pair of a batch for the same few windows at once, each key several times side by
+    side and far apart: each key stored once, the empty slots of a window behind all others;
+    counts of a counting table exact."""
+    from paper_2009_07914_gb300 import api
+    n = int(windows * W * 0.97)
+    keys, _ = _inputs(kb, n, windows + W)
+    batch = np.concatenate([np.repeat(keys, copies), np.tile(keys, copies)])
+    vals = np.arange(batch.size).astype(keys.dtype)
+    t = wc.SingleValueTable(kb, kb, min_capacity=windows * W, window_width=W, seed=SEED)
+    c = wc.CountingTable(kb, min_capacity=windows * W, window_width=W, seed=SEED)
+    for _ in range(3):
+        t.clear()
+        assert t.insert(batch, vals) == wc.WC_FLAG_DUPLICATE_KEY and t.size() == n
+        out, found, _ = t.retrieve(keys)
+        assert found.all()
+        np.testing.assert_array_equal(batch[out.astype(np.int64)], keys)  # one of the key's values
+        _layout(wc, t, 0)
+        dump = api.wc_table_dump_slots(t.handle).view(np.uint64)
+        k = (dump & np.uint64(0xFFFFFFFF) if kb == 4 else dump[::2]).reshape(-1, W)
+        empty = k == 0
+        assert (empty[:, 1:] >= empty[:, :-1]).all()
+        c.clear()
+        c.insert(batch)
+        assert c.size() == n
+        got, found, _ = c.retrieve(keys)
+        assert found.all() and (got == 2 * copies).all()
+
+
+@pytest.mark.parametrize("kb,W", [(4, 8), (8, 4)])
+def test_free_slots_with_other_words(wc, kb, W):
+    """A slot is free by its key: an empty slot or a tombstone whose value word is not what
+    clears and erases leave (left by a user kernel; written here by a copy) is claimed."""
+    import ctypes
+
+    import torch
+    from paper_2009_07914_gb300 import api
+    t = wc.SingleValueTable(kb, kb, min_capacity=5 * W, window_width=W, seed=SEED)
+    cap, tomb = t.capacity, 2 ** (8 * kb) - 1
+    words = np.zeros((cap, 2), np.uint32 if kb == 4 else np.uint64)
+    words[:, 1] = 9
+    words.reshape(-1, W, 2)[:, : W // 2, 0] = tomb  # each window: tombstones, then empty slots
+    src = torch.from_numpy(words.view(np.int32 if kb == 4 else np.int64)).cuda()
+    torch.cuda.synchronize()
+    rt = ctypes.CDLL("libcudart.so.13")  # the runtime instance libwc.so is linked against
+    assert rt.cudaMemcpy(ctypes.c_void_p(api.wc_table_device_view(t.handle).slots), ctypes.c_void_p(src.data_ptr()),
+                         ctypes.c_size_t(words.nbytes), 3) == 0
+    keys, vals = _inputs(kb, cap, 0x3F)
+    assert t.insert(np.repeat(keys, 3), np.repeat(vals, 3)) == wc.WC_FLAG_DUPLICATE_KEY and t.size() == cap
+    out, found, _ = t.retrieve(keys)
+    assert found.all()
+    np.testing.assert_array_equal(out, vals)
