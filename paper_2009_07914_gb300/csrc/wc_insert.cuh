@@ -19,9 +19,9 @@
 // table want the first slots of its windows at once.  A pair that loses one tries the next of
 // the window with another CAS and nothing read in between; reading window and slot again for
 // each lost race was slower than the group engine.  131,072 pairs of 4+4 bytes, load 0.6, that
-// engine / read again / next slot 18.8 / 21.6 / 14.6 us, at 0.9 32.4 / 35.4 / 27.4; 2^20 at
-// 0.9 55.9 / 53.3 / 52.0; 1000 at 0.6 14.8 / 15.2 / 8.6; sets of 8-byte keys, 222,476 at 0.9
-// 34.7 / 39.7 / 33.2.
+// engine / read again / next slot 18.8 / 21.6 / 12.8 us, at 0.9 32.4 / 35.4 / 26.3; 2^20 at
+// 0.9 55.9 / 53.3 / 48.7; 1000 at 0.6 14.8 / 15.2 / 8.6; sets of 8-byte keys, 222,476 at 0.9
+// 34.7 / 39.7 / 31.2.
 #pragma once
 
 #include "wc_launch.cuh"
@@ -261,23 +261,16 @@ __global__ void __launch_bounds__(kLookThreads, 4)
   flush_delta(t.size, added);
 }
 
-// Batches of 2^16 to 2^21 pairs in input order run three blocks per SM, two in tables below
-// 100,000 windows: with more, the pairs in flight outnumber the windows, and what is lost in
-// races for slots is more than the latency hidden (4+4 bytes; 2 / 3 / 5 blocks: 2^18 pairs at
-// load 0.9 47.8 / 59 / 68.7 us, at 0.5 30 / 36 / 38; 2^20 at 0.9 71.7 / 62.4 / 77.0, at 0.5
-// 44.4 / 36.5 / 45.8; 2^22 at 0.9 129 with three, 121 with four).
-inline int insert_blocks_per_sm(const wc_table* t, int most, uint64_t n, bool swept) {
-  if (swept || n <= (1ull << 16) || n >= (1ull << 21)) return most;
-  return std::min(most, t->windows < 100000 ? 2 : 3);
-}
-
+// As many blocks as fit, at every size: with fewer, so that fewer pairs race for slots, batches
+// of 2^17 to 2^21 pairs took longer (two or three blocks an SM against four, load 0.9: 222,476
+// pairs of 4+4 bytes 31.3 / 29.2 us, 600,000 45.3 / 40.3, 2^20 52.0 / 48.7; 317,816 8-byte
+// set keys at 0.6 20.7 / 18.8).
 template <class L, int W>
 cudaError_t insert_launch(const wc_table* t, const typename L::Key* keys, const typename L::Val* vals, uint64_t n,
                           unsigned long long* counter, const unsigned long long* n_dev, cudaStream_t s) {
   auto kern = counter != nullptr ? k_insert<L, W, true> : k_insert<L, W, false>;
-  const int per_sm = insert_blocks_per_sm(t, occupancy(kern, kLookThreads), n, counter != nullptr);
   const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
-  const uint64_t most = static_cast<uint64_t>(per_sm) * t->sm_count;
+  const uint64_t most = static_cast<uint64_t>(occupancy(kern, kLookThreads)) * t->sm_count;
   return launch_k(t, kern, static_cast<unsigned>(std::min(want, most)), kLookThreads, 0, s, desc_of(t), keys, vals, n,
                   counter, n_dev);
 }
