@@ -423,12 +423,25 @@ __global__ void __launch_bounds__(kPartThreads, 3) k_unsplit(const uint16_t* __r
 
 // ---- host side ---------------------------------------------------------------------------
 
+// Lookups in input order run as many blocks as fit (five an SM) while the table stays within
+// reach of the L2, three above 160 MiB: their window reads then come from DRAM, and with all
+// five in flight those get in each other's way.  Five against three blocks, queries all
+// present / half absent: 140 MiB of 4+4-byte slots at load 0.6 138 / 149 us against 155 / 161,
+// 200 MiB of 8+8 at 0.9 316 / 531 against 295 / 514, 430 MiB 878 / 1604 against 772 / 1451,
+// 500 MiB of 4+4 at 0.6 895 / 954 against 834 / 888; above 1 GiB and on Zipf queries the two
+// are within 2 % of each other.  (Two blocks: 2 to 5 % slower below 300 MiB, the same above.)
+constexpr uint64_t kLookFewer = 160ull << 20;
+inline int look_blocks_per_sm(const wc_table* t, int most, bool swept) {
+  return swept || t->table_bytes <= kLookFewer ? most : std::min(most, 3);
+}
+
 template <class L, int W, class Emit, class KIn = typename L::Key>
 cudaError_t lookup_launch(const wc_table* t, const KIn* keys, uint64_t n, unsigned long long* counter,
                           const Emit& emit, cudaStream_t s) {
   auto kern = counter != nullptr ? k_lookup<L, W, Emit, KIn, true> : k_lookup<L, W, Emit, KIn, false>;
   const uint64_t want = (n + kLookThreads - 1) / kLookThreads;
-  const uint64_t most = static_cast<uint64_t>(occupancy(kern, kLookThreads)) * t->sm_count;
+  const int per_sm = look_blocks_per_sm(t, occupancy(kern, kLookThreads), counter != nullptr);
+  const uint64_t most = static_cast<uint64_t>(per_sm) * t->sm_count;
   return launch_k(t, kern, static_cast<unsigned>(std::min(want, most)), kLookThreads, 0, s, desc_of(t), keys, n,
                   counter, emit);
 }
