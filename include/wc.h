@@ -227,8 +227,9 @@ typedef struct {
  * BLOCKED for those inserts when the batch holds at least 2^18 pairs and the table is
  * larger than 64 MiB, for lookups (wc_retrieve, wc_contains; hash sets too; and the counts of
  * multi-value tables with windows of at most 64 bytes) when the slots
- * take more than 512 MiB and the batch holds at least one query per 64 bytes of them (and
- * the stream is not being captured and the scratch fits), DIRECT otherwise.
+ * take more than 512 MiB and the batch holds at least one query per 64 bytes of them, and
+ * 2^24 of 8-byte keys (and the stream is not being captured and the scratch fits), DIRECT
+ * otherwise.
  * WC_SCHEME_DEDUP (lookups of single-value, counting and hash-set tables: wc_retrieve,
  * wc_contains): direct probing, but equal keys among each 32 consecutive queries of a
  * warp are found with one warp vote (__match_any_sync) and probed once, the result written

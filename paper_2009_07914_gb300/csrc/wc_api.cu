@@ -332,19 +332,28 @@ cudaError_t scratch_release(const wc_table* t, cudaStream_t s) {
 }
 
 // Lookups split by region where the table is far larger than L2 and the batch asks for each
-// of its 64-byte windows about once: the split costs ~9 ps a query (4-byte keys) and one
-// sequential pass over the table, and saves a random HBM line per query.  4+4-byte pairs at
-// load 0.9, half the queries absent, direct against split: 1.1 GiB table 28.5 against 46.3
-// G lookups/s for 2^27 queries, 27.8 against 30.1 for 2^24, 17.9 against 11.6 for 2^20;
-// 2 GiB table at load 0.5 37.0 against 34.2 for 2^24.  Between L2's size and 512 MiB the split
-// still wins on uniform queries (284 MiB, 2^26: 40.0 against 49.2) but loses on skewed ones,
-// whose hot lines stay in L2 (256 MiB, Zipf: 78 against 49); above, it wins both (1.1 GiB,
-// Zipf: 32.5 against 48.1).  8+8-byte pairs: 2.2 GiB 23.8 against 27.1, Zipf 28.8 against
-// 35.8.  (The splits in regions of 32 MiB; with those of look_region_mib and the faster
-// scatter 55.8 instead of 46.3.)  Not inside a stream capture: the scratch must not belong
-// to the graph.
+// of its 64-byte windows about once; with 8-byte keys only from 2^24 queries on.  The split
+// costs some 40 us, ~9 ps a query (4-byte keys; ~14 of 8 bytes) and one sequential pass over
+// the table, and saves a random HBM line per query.  Direct against split, microseconds,
+// queries all present / half absent / Zipf (one GB300):
+//   520 MiB, load 0.5, 8.7 M queries     4+4 bytes 199 / 207 / 169   222 / 229 / 174
+//                                        8+8 bytes 221 / 239 / 174   266 / 276 / 200
+//   520 MiB, load 0.5, 2^24 queries      4+4 bytes 360 / 370 / 316   333 / 341 / 296
+//                                        8+8 bytes 379 / 405 / 318   405 / 431 / 353
+//   the same, 3 * 2^23 queries           4+4 bytes 534 / 547 / 466   424 / 436 / 432
+//                                        8+8 bytes 559 / 601 / 473   496 / 546 / 512
+//   520 MiB, load 0.95, 2^24 queries     4+4 bytes 524 / 1213 / 351  478 / 1064 / 328
+//                                        8+8 bytes 648 / 1702 / 440  633 / 1575 / 437
+//   1.1 GiB, load 0.95, 18 M queries     4+4 bytes 672 / 1578 / 431  601 / 1304 / 354
+//   2.2 GiB, load 0.95, 36 M queries     8+8 bytes 1724 / 4707 / 1133  1622 / 3885 / 804
+//   SoA, 280 + 280 MiB, load 0.5, 36 M   4+4 bytes 1425 / 1099 / 883  664 / 654 / 751
+// Between L2's size and 512 MiB the split still wins on uniform queries (284 MiB, 2^26: 40.0
+// against 49.2 G/s, 32 MiB regions) but loses on skewed ones, whose hot lines stay in L2
+// (256 MiB, Zipf: 78 against 49).  Not inside a stream capture: a lookup takes no scratch by
+// itself there.
 bool lookup_splits(const wc_table* t, uint64_t n) {
-  return t->table_bytes > (512ull << 20) && n >= t->table_bytes / 64;
+  const uint64_t least = t->cfg.key_bytes == 8 ? 1ull << 24 : 0;
+  return t->table_bytes > (512ull << 20) && n >= t->table_bytes / 64 && n >= least;
 }
 
 int lookup_scheme(const wc_table* t, uint64_t n, cudaStream_t s) {
