@@ -195,7 +195,7 @@ typedef struct {
  * keys per thread); blocks_per_sm = resident blocks per SM the grid is
  * sized for (0 = the occupancy limit); scheme = how a bulk call visits the table
  * (WC_SCHEME_*); region_mib = table MiB per region of the blocked scheme (0 = 32, for
- * lookups of tables of up to 2 GiB 16; a region holds a power of two of windows, the most
+ * lookups of up to 2 GiB of slots -- of struct-of-arrays tables their keys -- 16; a region holds a power of two of windows, the most
  * that fit in region_mib MiB);
  * keys_in_flight = keys each group probes at once (1 or 2; 0 = 1): with 2, every trip of
  * a group loads the windows of two keys, so twice as many random window reads are in

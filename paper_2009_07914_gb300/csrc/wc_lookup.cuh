@@ -151,8 +151,8 @@ __device__ __forceinline__ Probe<L> probe_window(const typename L::Slot* slots, 
 // do not get back: 2^28 Zipf queries of 8+8 bytes over 4.8 GiB sweep in 2.89 ms with 32 and
 // 512 (3.07 with 256) and 2.84 with 16, for 0.6 ms more before and after.
 constexpr uint64_t kSmallSweep = 2ull << 30;
-__host__ __device__ constexpr int look_region_mib(uint64_t table_bytes) { return table_bytes > kSmallSweep ? 32 : 16; }
-__host__ __device__ constexpr uint32_t look_chunk(uint64_t table_bytes) { return table_bytes > kSmallSweep ? 512 : 256; }
+__host__ __device__ constexpr int look_region_mib(uint64_t slots_bytes) { return slots_bytes > kSmallSweep ? 32 : 16; }
+__host__ __device__ constexpr uint32_t look_chunk(uint64_t slots_bytes) { return slots_bytes > kSmallSweep ? 512 : 256; }
 
 // A warp's blocks of 32 consecutive inputs (warp-uniform).  kSwept: chunks of inputs are taken
 // from a counter in order, so the grid sweeps the batch front to back; otherwise the blocks
@@ -459,7 +459,8 @@ struct QuerySplit {
 template <class K, class V>
 cudaError_t query_split(const wc_table* t, int region_mib, const K* keys, uint64_t n, cudaStream_t s,
                         QuerySplit<K, V>& q) {
-  const RegionMap m = region_map(t, region_mib > 0 ? region_mib : look_region_mib(t->table_bytes));
+  const uint64_t slots_bytes = t->windows * t->W * t->slot_bytes;
+  const RegionMap m = region_map(t, region_mib > 0 ? region_mib : look_region_mib(slots_bytes));
   q.R = m.R;
   const uint64_t ntiles = (n + kPartTile - 1) / kPartTile;
   const uint64_t rv_bytes = align256(n * sizeof(V)), rf_bytes = align256(n);
