@@ -184,9 +184,13 @@ cudaError_t count_insert(const wc_table* t, const void* keys, const void* weight
   const uint64_t kb = static_cast<uint64_t>(t->cfg.key_bytes);
   const bool split = scheme_for(t, WC_OP_INSERT, n) == WC_SCHEME_BLOCKED;
   const uint64_t skip = split ? kSplitHeader + 2 * ((n * kb + 255) / 256 * 256) : 0;
-  // windows of at most 64 bytes: their insert takes a batch size from the device (a small
-  // batch is not worth the launch that zeroes it)
-  const bool dense = n >= (1ull << 18) && t->W * t->slot_bytes <= 64;
+  // Windows of at most 64 bytes: their insert takes a batch size from the device.  From 2^19
+  // inputs on the shorter list of a skewed batch is worth the zeroed cursor and the tiles'
+  // atomics on it.  Padded against dense, Zipf / uniform draws, 4-byte keys: 270,000 over 9 M
+  // 51 / 71 against 55 / 75 us, 600,000 60 / 81 against 59 / 85, 2^22 over 10^6 96 / 177
+  // against 80 / 182; 8-byte keys: 290,000 uniform, 16 of each, 64 against 68, 600,000 over
+  // 4.5 M 80 / 91 against 75 / 95, 2^22 over 10^6 206 / 305 against 192 / 307.
+  const bool dense = n >= (1ull << 19) && t->W * t->slot_bytes <= 64;
   const void* ak = nullptr;
   const void* av = nullptr;
   const unsigned long long* n_dev = nullptr;
