@@ -10,7 +10,10 @@
  * (or the one the caller fixes), a table of the caller's kind, widths and options is
  * filled to the given load with `sample_keys` distinct keys, and every valid group size
  * of insert, retrieve (and keys in flight 1 or 2 where the lookup kernel supports it) and
- * erase is timed with CUDA events (best of three calls).  A lookup is timed on two query
+ * erase is timed with CUDA events (best of three calls); inserts and lookups of windows of at
+ * most 64 bytes run one key per thread and are timed in their one shape, and lookups in
+ * input order, as the sample's table is below the size from which they are split (wc.h).  A
+ * lookup is timed on two query
  * streams: uniform keys, half of them absent (bound by HBM), and queries over a hot 1/64 of
  * the keys (bound by L2, as a skewed stream's hot keys are); a shape has to serve both.
  * W is the one with the smallest insert + retrieve time.  A shape or width replaces the

@@ -189,7 +189,9 @@ class Tuner {
 
   // Time the table's default shape of `op` and every other valid group size (and, for
   // lookups whose lanes hold at most 32 bytes of window, two keys in flight); keep the
-  // default unless the fastest other shape beats it by more than 10 %.
+  // default unless the fastest other shape beats it by more than 10 %.  Inserts into and
+  // lookups of windows of at most 64 bytes run one key per thread whatever the shape says:
+  // they are timed once.
   template <class Prep, class Op>
   wc_status sweep(wc_table* t, int W, int op, Prep prep, Op timed, WindowResult& r) {
     wc_launch def{};
@@ -197,7 +199,8 @@ class Tuner {
     if (st != WC_OK) return st;
     const int def_k = std::max(1, def.keys_in_flight);
     std::vector<wc_launch> cands{def};
-    for (int g = 1; g <= W && g <= 32; g *= 2) {
+    const bool shaped = op == WC_OP_ERASE || W * slot_bytes() > 64;
+    for (int g = 1; shaped && g <= W && g <= 32; g *= 2) {
       for (int k = 1; k <= 2; ++k) {
         if (k == 2 && (op != WC_OP_RETRIEVE || is_set() || (W / g) * slot_bytes() > 32)) continue;
         if (g == def.group_size && k == def_k) continue;

@@ -31,6 +31,7 @@ SHAPES = {  # slot bytes -> W -> valid lanes per key
     16: {2: [1, 2], 4: [1, 2, 4], 8: [1, 2, 4, 8], 16: [4, 8, 16]},
 }
 BLOCKS = (256, 128)
+ONE_KEY_PER_THREAD = 64  # windows of at most this many bytes: inserts and lookups have one launch shape
 
 
 def _cache_path() -> str:
@@ -90,7 +91,8 @@ def tune_table(h: int, keys: torch.Tensor, values: torch.Tensor, queries: torch.
     out = torch.empty(queries.numel(), dtype=torch.int32 if vb == 4 else torch.int64, device=keys.device)
     found = torch.empty(queries.numel(), dtype=torch.uint8, device=keys.device)
     for opname, op in (("insert", WC_OP_INSERT), ("retrieve", WC_OP_RETRIEVE), ("erase", WC_OP_ERASE)):
-        kif = api.wc_table_get_launch(h, op)["keys_in_flight"]  # kept as the table has it
+        lc = api.wc_table_get_launch(h, op)
+        kif = lc["keys_in_flight"]  # kept as the table has it
         key = cache_key(kb, vb, W, alpha, n, opname)
         if key in cache:
             c = cache[key]
@@ -99,8 +101,9 @@ def tune_table(h: int, keys: torch.Tensor, values: torch.Tensor, queries: torch.
             continue
         schemes = [WC_SCHEME_DIRECT, WC_SCHEME_BLOCKED] if opname == "insert" else [WC_SCHEME_DIRECT]
         results = []
-        for G in SHAPES[sb][W]:
-            for blk in BLOCKS:
+        shaped = op == WC_OP_ERASE or W * sb > ONE_KEY_PER_THREAD
+        for G in SHAPES[sb][W] if shaped else [lc["group_size"]]:
+            for blk in BLOCKS if shaped else [lc["block_threads"]]:
                 for sc in schemes:
                     api.wc_table_set_launch(h, op, G, blk, 0, sc, 0, kif)
                     if opname == "insert":
@@ -169,24 +172,39 @@ def recommend_window(kb: int, vb: int, n: int, alpha: float, reps: int = 3, repo
 
 # Lanes per key the batched executor is built for (wc_exec.h): window width -> (insert, lookup).
 EXEC_SHAPES = {4: ([1, 2], [1, 2]), 8: ([1, 2, 4], [1, 2, 4]), 16: ([2, 4], [2, 4])}
+EXEC_DEFAULT_INSERT = {4: 1, 8: 2}
 
 
 def executor_groups(W: int, n: int = 1 << 22, alpha: float = 0.75, reps: int = 3, use_cache: bool = True,
                     report=None) -> dict:
-    """Lanes per key for the batched executor's inserts and lookups (wc_executor_config
-    group_insert / group_retrieve) on 4+4-byte tables of window width W: the executor
-    cuts work into tiles and never region-splits, so the candidates are timed with the
-    direct scheme on a seeded sample of n keys at load alpha.  Cached like tune_table."""
+    """Lanes per key for the batched executor (wc_executor_config group_insert /
+    group_retrieve) on 4+4-byte tables of window width W: the executor cuts work into tiles
+    and never region-splits, so the candidates are timed with the direct scheme on a seeded
+    sample of n keys at load alpha.  Windows of at most 64 bytes are filled and looked up one
+    key per thread: group_insert is the executor's default there and group_retrieve, which only
+    erases take, is timed on erases.  Cached like tune_table."""
     keys, values, queries = sample(4, n)
     cache = _load_cache() if use_cache else {}
     gi_set, gr_set = EXEC_SHAPES[W]
+    lean = W * 8 <= ONE_KEY_PER_THREAD
     h = api.wc_table_create(0, 4, 4, int(math.ceil(n / alpha)), W, 0, 0x5EED, torch.cuda.current_device())
     s = torch.cuda.current_stream()
     out = torch.empty(queries.numel(), dtype=torch.int32, device=keys.device)
     found = torch.empty(queries.numel(), dtype=torch.uint8, device=keys.device)
     best = {}
+    ops = [("exec_erase", WC_OP_ERASE, gr_set)] if lean else [("exec_insert", WC_OP_INSERT, gi_set),
+                                                              ("exec_retrieve", WC_OP_RETRIEVE, gr_set)]
+
+    def fill():
+        api.wc_table_clear(h, s)
+        api.wc_insert(h, keys, values, n, s)
+
+    def fill_and_erase():  # the same insert for every candidate
+        fill()
+        api.wc_erase(h, keys, n, s)
+
     try:
-        for opname, op, gset in (("exec_insert", WC_OP_INSERT, gi_set), ("exec_retrieve", WC_OP_RETRIEVE, gr_set)):
+        for opname, op, gset in ops:
             key = cache_key(4, 4, W, alpha, n, opname)
             if key in cache:
                 best[opname] = cache[key]
@@ -194,27 +212,23 @@ def executor_groups(W: int, n: int = 1 << 22, alpha: float = 0.75, reps: int = 3
             res = []
             for G in gset:
                 api.wc_table_set_launch(h, op, G, 256, 0, WC_SCHEME_DIRECT, 0)
-                if op == WC_OP_INSERT:
-                    def f():
-                        api.wc_table_clear(h, s)
-                        api.wc_insert(h, keys, values, n, s)
-                    ms = _time(f, reps)
-                else:
-                    ms = _time(lambda: api.wc_retrieve(h, queries, out, found, queries.numel(), s), reps)
-                res.append({"op": opname, "W": W, "group": G, "ms": ms})
+                f = {WC_OP_INSERT: fill, WC_OP_ERASE: fill_and_erase,
+                     WC_OP_RETRIEVE: lambda: api.wc_retrieve(h, queries, out, found, queries.numel(), s)}[op]
+                res.append({"op": opname, "W": W, "group": G, "ms": _time(f, reps)})
                 if report:
                     report(res[-1])
             best[opname] = min(res, key=lambda r: r["ms"])
             cache[key] = best[opname]
             if op == WC_OP_INSERT:  # lookups need the table filled
                 api.wc_table_set_launch(h, op, best[opname]["group"], 256, 0, WC_SCHEME_DIRECT, 0)
-                api.wc_table_clear(h, s)
-                api.wc_insert(h, keys, values, n, s)
+                fill()
     finally:
         torch.cuda.synchronize()
         api.wc_table_destroy(h)
     if use_cache:
         _save_cache(cache)
+    if lean:
+        return {"group_insert": EXEC_DEFAULT_INSERT[W], "group_retrieve": best["exec_erase"]["group"]}
     return {"group_insert": best["exec_insert"]["group"], "group_retrieve": best["exec_retrieve"]["group"]}
 
 

@@ -197,3 +197,27 @@ def test_window_zero_without_tuning_is_the_64_byte_window(monkeypatch):
     m = wc.MultiValueTable(4, 4, min_capacity=4096, value_pool_capacity=1 << 14)
     assert m.info["window_width"] == 4
     m.close()
+
+
+def test_shapes_that_launch_the_same_kernel_are_timed_once(tmp_path, monkeypatch):
+    """Inserts and lookups of windows of at most 64 bytes run one key per thread: both tuners
+    time them in one shape (and erases, and wider windows, in every one)."""
+    from paper_2009_07914_gb300 import build
+    build.build()
+    monkeypatch.setenv("WC_TUNE_CACHE", str(tmp_path / "cache.json"))
+    from paper_2009_07914_gb300 import api, tune
+    for kb, W, groups in ((4, 4, 3), (4, 8, 4), (8, 2, 2), (8, 4, 3)):
+        a = api.wc_autotune(0, kb, kb, window_width=W, load=0.9, sample_keys=1 << 12, use_cache=False)
+        assert a["candidates"] == 2 + groups
+    assert api.wc_autotune(0, 4, 4, window_width=16, load=0.9, sample_keys=1 << 12, use_cache=False)["candidates"] > 12
+    n = 1 << 12
+    keys, values, queries = tune.sample(4, n)
+    h = api.wc_table_create(0, 4, 4, int(n / 0.9) + 1, 8, 0, 0x5EED, 0)
+    seen = []
+    tune.tune_table(h, keys, values, queries, reps=1, use_cache=False, report=seen.append)
+    api.wc_table_destroy(h)
+    per_op = {op: len({(r["group"], r["block"]) for r in seen if r["op"] == op}) for op in ("insert", "retrieve", "erase")}
+    assert per_op == {"insert": 1, "retrieve": 1, "erase": 8}
+    seen = []
+    g = tune.executor_groups(8, n=n, reps=1, use_cache=False, report=seen.append)
+    assert g["group_insert"] == 2 and [r["op"] for r in seen] == ["exec_erase"] * 3
