@@ -510,10 +510,11 @@ def run_wc(args, rank, world, local_rank):
         "vs_baseline": None, "dtype": "u32", "data": "synthetic",
         "config": {"workload": workload_name, "n": n, "queries": n, "present_fraction": 0.5,
                    "capacity": info["capacity"], "achieved_alpha": n / info["capacity"],
-                   "window_slots": info["window_width"], "tuning": tuning, "group_insert": g_ins,
-                   "group_retrieve": g_ret,
-                   "insert_keys_in_flight": api.wc_table_get_launch(h, wc.WC_OP_INSERT)["keys_in_flight"],
-                   "retrieve_keys_in_flight": api.wc_table_get_launch(h, wc.WC_OP_RETRIEVE)["keys_in_flight"],
+                   "window_slots": info["window_width"], "tuning": tuning, "group_insert": 1 if narrow else g_ins,
+                   "group_retrieve": 1 if narrow else g_ret,
+                   "insert_keys_in_flight":
+                       1 if narrow else api.wc_table_get_launch(h, wc.WC_OP_INSERT)["keys_in_flight"],
+                   "retrieve_keys_in_flight": 1 if narrow else kif_ret,
                    "retrieve_scheme": {0: "auto", 1: "direct", 2: "region split", 3: "grouped duplicates"}[
                        api.wc_table_get_launch(h, wc.WC_OP_RETRIEVE)["scheme"]],
                    "table_bytes": info["table_bytes"], "overflow_bits": bool(info["options"] & 1),
