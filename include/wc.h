@@ -195,15 +195,17 @@ typedef struct {
  * keys per thread); blocks_per_sm = resident blocks per SM the grid is
  * sized for (0 = the occupancy limit); scheme = how a bulk call visits the table
  * (WC_SCHEME_*); region_mib = table MiB per region of the blocked scheme (0 = 32, for
- * lookups of up to 2 GiB of slots -- of struct-of-arrays tables their keys -- 16; a region holds a power of two of windows, the most
- * that fit in region_mib MiB);
+ * lookups of up to 2 GiB of slots -- of struct-of-arrays tables their keys -- 16; a region
+ * holds a power of two of windows, the most that fit in region_mib MiB);
  * keys_in_flight = keys each group probes at once (1 or 2; 0 = 1): with 2, every trip of
  * a group loads the windows of two keys, so twice as many random window reads are in
  * flight per warp (single-value retrieves of up to 32 bytes of window per lane; elsewhere
  * it is taken as 1).  Default 2 for lookups of 4+4-byte single-value tables, else 1.
  * Inserts into and lookups of windows of at most 64 bytes run one key per thread, whatever
  * group_size, block_threads, blocks_per_sm and keys_in_flight say (WC_SCHEME_DEDUP keeps the
- * group); erases, wider windows and multi-value tables take them as they are. */
+ * group); so do the counts of multi-value tables with such windows and the swept inserts of
+ * open-addressing ones.  Erases, wider windows and the other calls of multi-value tables take
+ * them as they are. */
 typedef struct {
   int32_t group_size;
   int32_t block_threads;

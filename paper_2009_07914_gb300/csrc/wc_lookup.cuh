@@ -206,7 +206,7 @@ struct BatchBlocks {
     const uint64_t a = (c * ratio >> 16 & ~127ull) + kSweepLead;
     uint64_t e = ((c + stride) * ratio >> 16 & ~127ull) + kSweepLead;
     if (e > tab_bytes) e = tab_bytes;
-    if (a < e)  // at most 16 KiB
+    if (a < e)  // at most 32 KiB: 512 inputs of up to 64 bytes of table each
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(tab + a), "r"(static_cast<uint32_t>(e - a))
                    : "memory");
   }

@@ -69,7 +69,7 @@ cudaError_t sv_insert_op(const wc_table* t, const void* keys, const void* vals, 
   RegionSplit<Key, Val> sp;
   const RegionMap m = region_map(t, lc.region_mib);
   cudaError_t e = v != nullptr ? region_split(t, m, k, v, n, s, sp, 0, 0, n_dev)
-                               : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp);
+                               : region_split<Key, Val, kValsNone>(t, m, k, nullptr, n, s, sp, 0, 0, n_dev);
   if (e == cudaSuccess) e = insert_kernel<L, G, S, H>(t, sp.keys, sp.vals, n, sp.counters, s, n_dev);
   const cudaError_t r = scratch_release(t, s);
   return e != cudaSuccess ? e : r;
