@@ -121,7 +121,7 @@ cudaError_t sv_run(const wc_table* t, int op, const void* keys, const void* vals
   auto kern = k_sv_erase<L, G, S, H>;
   const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : occupancy(kern, block);
   const EngineGrid g = engine_grid(n, G, block, bps, t->sm_count);
-  return launch_k(t, kern, g.blocks, block, 0, s, d, k, n, g.per_warp);
+  return launch_k(t, kern, g.blocks, block, 0, s, d, k, n, erase_chunk(g.per_warp));
 }
 
 }  // namespace wc

@@ -673,6 +673,11 @@ __device__ __forceinline__ void sv_erase_range(const TableDesc& t, const KIn* __
   bool act = false;
   Key k = 0;
   uint32_t w = 0, step = 0, j = 0, tag = 0, h = 0;
+  // Half-line reads in front of the CAS (kClaim, wc_device.cuh) up to about the L2's size, whole
+  // lines above: 2^22 keys of 8-byte sets erased in 55 MB 60 -> 46 us, 2^22 of 8+8 bytes in 111
+  // MB 59 -> 51, but 2^24 of 4+4 in 149 MB 229 -> 248, in 223 MB 229 -> 254 (the same from 450 MB).
+  constexpr uint64_t kWindowBytes = static_cast<uint64_t>(W) * (L::kHalf ? 4 : L::kWords * 8);
+  const bool claim = t.p * kWindowBytes <= (128ull << 20);
   Feed<KIn> fk;
   while (true) {
     const bool more = src.ensure();
@@ -703,7 +708,8 @@ __device__ __forceinline__ void sv_erase_range(const TableDesc& t, const KIn* __
     uint32_t mm = 0, me = 0, mt = 0;
     const uint64_t lane_slot = static_cast<uint64_t>(w) * W + Steps<H>::offset(h, SW) + ln.r * S;
     if (act) {
-      load_slots<L, S, true>(slots + lane_slot, s);
+      if (claim) load_slots<L, S, true>(slots + lane_slot, s);
+      else load_slots<L, S>(slots + lane_slot, s);
       classify<L, S>(s, k, mm, me, mt);
     }
     const uint32_t bm = group_vote<G>(mm != 0, ln.gbase);
@@ -742,10 +748,29 @@ struct NoOnErase {
   __device__ void operator()(const Slot&) const {}
 };
 
+// Chunks strided over the warps, about eight each (all of a warp's keys in one where they are
+// few): one-key-per-thread inserts take a batch front to back, so its last keys sit furthest
+// along their sequences, and of keys erased in the order they were inserted the warp with the
+// last consecutive range would be the last to end (half of 2^22 pairs of 4+4 bytes at load 0.9,
+// two lanes per key 101 -> 79 us, of 2^25 one lane 698 -> 596 and two 717 -> 606; of 2^26 of 8+8
+// bytes 1998 -> 1844).
+inline uint32_t erase_chunk(uint64_t per_warp) {
+  if (per_warp <= 64) return static_cast<uint32_t>(std::max<uint64_t>(per_warp, 1));
+  return static_cast<uint32_t>((per_warp + 255) / 256 * 32);
+}
+// Blocks per SM that the erase kernel has to leave room for: what it had with one consecutive
+// range per warp.  The strided chunks' registers would cost one of them (two lanes, load 0.6,
+// 2^23 pairs of 4+4 bytes 117 -> 107 us, of 8+8 bytes 190 -> 150).
+template <class L, int G, int S>
+constexpr int erase_min_blocks() {
+  constexpr int words = L::kHalf ? S / 2 : S * L::kWords;  // 64-bit words of slots per lane
+  return words <= 2 ? 6 : words <= 4 || (G == 1 && L::kWords == 1) ? 5 : 4;
+}
+
 template <class L, int G, int S, int H = 1>
-__global__ void __launch_bounds__(256) k_sv_erase(TableDesc t, const typename L::Key* __restrict__ keys, uint64_t n,
-                                                  uint64_t per_warp) {
-  RangeSrc src(n, per_warp, nullptr, 0);
+__global__ void __launch_bounds__(256, erase_min_blocks<L, G, S>()) k_sv_erase(TableDesc t, const typename L::Key* __restrict__ keys, uint64_t n,
+                                                  uint32_t chunk) {
+  RangeSrc src(StridedChunks{}, n, chunk);
   if (src.next >= src.end) return;
   uint32_t flags = 0;
   long long removed = 0;

@@ -170,3 +170,29 @@ def test_free_slots_with_other_words(wc, kb, W):
     out, found, _ = t.retrieve(keys)
     assert found.all()
     np.testing.assert_array_equal(out, vals)
+
+
+@pytest.mark.parametrize("kb,W,group", [(4, 8, 1), (4, 8, 4), (8, 4, 2), (4, 16, 2)])
+@pytest.mark.parametrize("n", [1, 33, 500_009, 700_001, 3_000_017])
+def test_erases_in_strided_chunks(wc, kb, W, group, n):
+    """Erased keys are gone, their neighbours stay and the size is exact, from batches that give
+    a warp a few keys to batches of several chunks a warp."""
+    import torch
+    from paper_2009_07914_gb300 import api
+    from paper_2009_07914_gb300.table import to_device
+    keys, vals = _inputs(kb, 2 * n + 64, n + kb)
+    t = wc.SingleValueTable(kb, kb, min_capacity=int(2 * n / 0.85) + 64, window_width=W, seed=SEED)
+    t.set_launch(wc.WC_OP_ERASE, group)
+    dev = torch.device("cuda", torch.cuda.current_device())
+    k, v = to_device(keys, kb, dev), to_device(vals, kb, dev)
+    api.wc_insert(t.handle, k[:2 * n], v[:2 * n])
+    gone = k[:2 * n:2].contiguous()
+    api.wc_erase(t.handle, gone)
+    api.wc_erase(t.handle, k[2 * n:])  # never stored
+    assert t.size() == n
+    out, found = torch.empty_like(k), torch.empty(k.numel(), dtype=torch.uint8, device=dev)
+    api.wc_retrieve(t.handle, k, out, found)
+    assert not found[:2 * n:2].any() and bool(found[1:2 * n:2].all()) and not found[2 * n:].any()
+    assert torch.equal(out[1:2 * n:2], v[1:2 * n:2])
+    api.wc_insert(t.handle, gone, gone)
+    assert t.size() == 2 * n and t.status() == 0
