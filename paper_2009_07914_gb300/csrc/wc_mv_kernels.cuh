@@ -372,7 +372,9 @@ __global__ void __launch_bounds__(kAggThreads, W <= 4 ? 1280 / kAggThreads : 1) 
       }
       // A hot key shows up as the warp's first one: its copies are counted by their lowest
       // lane.  The rest count one by one (grouping every key of the warp with
-      // __match_any_sync cost more than the atomics it saved).
+      // __match_any_sync cost more than the atomics it saved).  From how many copies on makes
+      // no difference (2, 4, 6, 10 or 16: within 1 % on 2^27 Zipf and uniform draws); never
+      // grouping costs 20 % where one key is all of the batch (2^24 pairs 178 -> 220 us).
       const unsigned long long first = __shfl_sync(kFull, key, 0);  // every lane shuffles
       uint32_t peers = __ballot_sync(kFull, valid && key == first);
       if (__popc(peers) < 6 || !((peers >> lane) & 1u)) peers = 1u << lane;
