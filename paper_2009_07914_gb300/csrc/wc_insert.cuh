@@ -11,7 +11,7 @@
 // walk has met an empty slot or its end.
 //
 // The sweep of 2^27 pairs, one GB300, that engine against this kernel (with half-line
-// reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.86 ms (2.63 with the table
+// reads): 4+4 bytes at load 0.9 with overflow bits 3.51 -> 2.97 ms (2.73 with the table
 // copied to L2 ahead of the sweep, BatchBlocks::prefetch), at 0.5 3.11 -> 2.30; 8+8 bytes at
 // 0.9 5.02 -> 4.35; sets of 8-byte keys at 0.9 4.6 -> 3.2.
 //

@@ -164,7 +164,7 @@ __host__ __device__ constexpr uint32_t look_chunk(uint64_t slots_bytes) { return
 // (early), so no warp waits for the counter.  Chunks of 192, 128 and 64: 1.47, 1.65 and 2.9
 // ms for 2^27 lookups, as the counter takes only some 0.3 to 0.7 atomics per ns.  It takes
 // fewest beside inserts, which are fastest with 512 asked for when needed (2^27 pairs of 4+4
-// bytes 2.63 ms, early 2.84, early 256 2.78; 2^26 Zipf counting inserts 0.63, early 256
+// bytes: early 8 % slower, early 256 6 %; 2^26 Zipf counting inserts 0.63 ms, early 256
 // 0.88).  Batches below 2^21 take shorter chunks: there are about 5000 warps.
 template <bool kSwept>
 struct BatchBlocks {
